@@ -6,10 +6,15 @@
 #include <cstring>
 #include <new>
 
+#include <vector>
+
 #include "sk_decomp.h"
+#include "sk_factors64.h"
 #include "sk_internal.h"
 
 namespace {
+
+using namespace sk;
 
 const char* g_create_error = "";
 thread_local std::string g_create_error_buf;
@@ -25,6 +30,17 @@ struct DeviceGuard {
     if (prev >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != prev) cudaSetDevice(prev);
   }
 };
+
+// The FP64 factor tables (136 KB), built once per process; every context
+// keeps a device copy.
+const char* factor_tables() {
+  static const std::vector<char> t = [] {
+    std::vector<char> v(F64_TABLES_BYTES);
+    f64_build_tables(v.data());
+    return v;
+  }();
+  return t.data();
+}
 
 int fail(sk_ctx* ctx, int code, const char* fmt, const char* detail = "") {
   char buf[512];
@@ -61,6 +77,7 @@ void carve_eval_buffers(Bump& bp, const EvalShape& s, EvalBufs& b) {
   b.n_chunks = s.n_chunks;
   b.pair_np = pair32_np(s.M);
   b.threads64 = s.threads64;
+  b.factors64 = s.factors64;
   b.fuse_finish = fp32 && s.fuse_finish;
   const int64_t nsort = s.N > s.M ? s.N : s.M;
   b.sort_blocks = sort_grid_blocks(nsort > 0 ? nsort : 1);
@@ -237,7 +254,10 @@ int sk_create(sk_ctx** out, int device, size_t workspace_bytes) {
       (e = cudaStreamCreateWithFlags(&ctx->aux_stream, cudaStreamNonBlocking)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&ctx->fork_ev, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaEventCreateWithFlags(&ctx->join_ev, cudaEventDisableTiming)) != cudaSuccess ||
-      (e = cudaMallocHost(&ctx->h_flags, 256)) != cudaSuccess) {
+      (e = cudaMallocHost(&ctx->h_flags, 256)) != cudaSuccess ||
+      (e = cudaMalloc(&ctx->factors64, F64_TABLES_BYTES)) != cudaSuccess ||
+      (e = cudaMemcpy(ctx->factors64, factor_tables(), F64_TABLES_BYTES,
+                      cudaMemcpyHostToDevice)) != cudaSuccess) {
     code = e == cudaErrorMemoryAllocation ? SK_ENOMEM : SK_ECUDA;
   } else if (workspace_bytes > 0) {
     if ((e = cudaMalloc(&ctx->ws, workspace_bytes)) != cudaSuccess)
@@ -273,6 +293,7 @@ void sk_destroy(sk_ctx* ctx) {
   free_membrane_ops(ctx);
   free_fmm_ops(ctx);
   if (ctx->ws) cudaFree(ctx->ws);
+  if (ctx->factors64) cudaFree(ctx->factors64);
   if (ctx->h_flags) cudaFreeHost(ctx->h_flags);
   for (int i = 0; i < 4; ++i)
     if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
@@ -397,6 +418,7 @@ int eval_entry(sk_ctx* ctx, int layer, int precision, int mem, int64_t N, const 
   s.mu = mu;
   s.copy_inputs = mem == SK_HOST;
   s.small_sort_points = ctx->small_sort_points;
+  s.factors64 = ctx->factors64;
   s.split_sorts = true;
   choose_decomposition(s, ctx->sm_count);
   const size_t need = eval_workspace_bytes(s);

@@ -218,6 +218,7 @@ EvalShape capsule_shape(const sk_capsule* c) {
     s.n_delta = c->n_delta;
   }
   s.small_sort_points = c->ctx->small_sort_points;
+  s.factors64 = c->ctx->factors64;
   s.split_sorts = true;  // the step graphs fork the target sort onto a second stream
   choose_decomposition(s, c->ctx->sm_count);
   return s;

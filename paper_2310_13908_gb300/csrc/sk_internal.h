@@ -163,6 +163,7 @@ struct EvalBufs {
   float4* srcLo = nullptr;        // double layer, FP32C: residual (y - c) - fl32(y - c) per source
   double4_32a* src64 = nullptr;       // FP64 packed sources (pos, density)
   double4_32a* nrm64 = nullptr;       // FP64 packed normals (double layer)
+  const char* factors64 = nullptr;    // FP64 factor tables (the context's)
   float4* segbox = nullptr;       // per segment: lo, hi
   int* tgt_perm = nullptr;        // sorted target -> original index
   float4* tgtF = nullptr;         // FP32 sorted targets: (x, y, z, 1/delta), (rc2, rt2, 0, 0)
@@ -217,6 +218,7 @@ struct sk_ctx {
   cudaStream_t aux_stream = nullptr;
   cudaEvent_t fork_ev = nullptr;
   cudaEvent_t join_ev = nullptr;
+  char* factors64 = nullptr;  // FP64 kernel factors of both layers (sk_factors64.h)
   char* ws = nullptr;
   size_t ws_bytes = 0;
   bool ws_fixed = false;
@@ -256,6 +258,7 @@ struct EvalShape {
   bool copy_inputs = false;  // inputs/outputs live in the workspace (host-memory calls)
   int n_chunks = 1;
   int threads64 = TPB64;  // CTA size of the FP64 pair kernel (TPB64 or TPB64_SMALL)
+  const char* factors64 = nullptr;  // SK_FP64: the context's factor tables
   bool fuse_finish = false;  // FP32C: finish target blocks inside the pair kernel
   // point sets of at most this many points are ordered by one single-block
   // kernel instead of fifteen launches (0: never)
