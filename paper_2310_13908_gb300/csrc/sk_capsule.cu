@@ -70,39 +70,6 @@ namespace {
 
 inline unsigned blocks(int64_t n) { return (unsigned)((n + 255) / 256); }
 
-// delta*_p = max over the nodes of patch p of the largest distance to an
-// existing grid neighbour (offsets a, b in {-1, 0, 1}) (Eq. regparam).
-__global__ void k_delta_star_patch(const double* __restrict__ X, int m,
-                                   unsigned long long* __restrict__ pmax) {
-  const int n = m - 1;
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  double best = 0.0;
-  int p = -1;
-  if (i < 6 * (int64_t)n * n) {
-    p = (int)(i / ((int64_t)n * n));
-    const int r = (int)(i % ((int64_t)n * n));
-    const int j = r / n, k = r % n;
-    const double x = X[3 * i], y = X[3 * i + 1], z = X[3 * i + 2];
-    for (int a = -1; a <= 1; ++a)
-      for (int b = -1; b <= 1; ++b) {
-        const int jj = j - a, kk = k - b;
-        if ((a == 0 && b == 0) || jj < 0 || jj >= n || kk < 0 || kk >= n) continue;
-        const int64_t q = (int64_t)p * n * n + (int64_t)jj * n + kk;
-        const double dx = x - X[3 * q], dy = y - X[3 * q + 1], dz = z - X[3 * q + 2];
-        best = fmax(best, sqrt(dx * dx + dy * dy + dz * dz));
-      }
-  }
-  // nonnegative doubles order like their bit patterns
-  if (p >= 0) atomicMax(pmax + p, (unsigned long long)__double_as_longlong(best));
-}
-
-__global__ void k_delta_fill(const unsigned long long* __restrict__ pmax, int m, double C,
-                             double* __restrict__ delta) {
-  const int n = m - 1;
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < 6 * (int64_t)n * n) delta[i] = C * __longlong_as_double((long long)pmax[i / ((int64_t)n * n)]);
-}
-
 // X += dt (u + u_inf(X)); background flows of Eqs. shear_flow, poiseuille_flow.
 __global__ void k_euler(double* __restrict__ X, const double* __restrict__ u, int64_t N, double dt,
                         sk_flow fl) {
@@ -248,9 +215,7 @@ void enqueue_velocity(sk_capsule* c, const double* P, int mode, const EvalShape&
     b.delta = us.delta;
   } else {
     if (c->auto_delta) {
-      cudaMemsetAsync(c->patch_max, 0, 8 * sizeof(unsigned long long), st);
-      k_delta_star_patch<<<blocks(c->N), 256, 0, st>>>(P, c->m, c->patch_max);
-      k_delta_fill<<<blocks(c->N), 256, 0, st>>>(c->patch_max, c->m, 1.0, c->delta);
+      enqueue_patch_delta(P, c->m - 1, c->patch_max, c->delta, st);
     }
     b.src_xyz = P;
     b.src_w = c->w;
@@ -302,9 +267,7 @@ void capsule_enqueue_step_inputs(sk_capsule* c, EvalBufs& b, cudaStream_t st, in
     enqueue_skalak(*op, c->X, c->ref6, c->Es, c->ED, c->f, c->w, st);
   }
   if (c->auto_delta) {
-    cudaMemsetAsync(c->patch_max, 0, 8 * sizeof(unsigned long long), st);
-    k_delta_star_patch<<<blocks(c->N), 256, 0, st>>>(c->X, c->m, c->patch_max);
-    k_delta_fill<<<blocks(c->N), 256, 0, st>>>(c->patch_max, c->m, 1.0, c->delta);
+    enqueue_patch_delta(c->X, c->m - 1, c->patch_max, c->delta, st);
   }
   b.src_xyz = c->X;
   b.src_w = c->w;

@@ -110,6 +110,15 @@ __device__ __forceinline__ void write_sl_record(float4* o, float x, float y, flo
   o[1] = make_float4(-z, -z, g0, g0);
   o[2] = make_float4(g1, g1, g2, g2);
 }
+// 1/sqrt(x): the hardware's approximation y0 (about 20 bits, one instruction)
+// and one step of Householder's cubic iteration, y0 (1 + e/2 + 3/8 e^2) with
+// e = 1 - x y0^2; the term left out is below 2^-60. Overflowed x gives 0.
+__device__ __forceinline__ double rsqrt_fp64(double x) {
+  double y0;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+  const double e = __double2hiint(x) < 0x7ff00000 ? fma(-x, y0 * y0, 1.0) : 0.0;
+  return fma(y0, e * fma(0.375, e, 0.5), y0);
+}
 #endif
 
 // Padding sources sit this far away, with zero density.
@@ -373,6 +382,10 @@ int membrane_upsampling(sk_ctx* ctx, MembraneOp* op);
 void enqueue_upsample(const MembraneOp& op, const double* X, const double* W, const double* f,
                       cudaStream_t st);
 UpsampledSources upsampled_sources(const MembraneOp& op);
+// delta* of Eq. regparam (C = 1) at the nodes X of six n x n patches, per
+// patch, into delta; pmax: 8 words of scratch.
+void enqueue_patch_delta(const double* X, int n, unsigned long long* pmax, double* delta,
+                         cudaStream_t st);
 void enqueue_area_volume(const MembraneOp& op, const double* X, double* out2, cudaStream_t st);
 void enqueue_moments(const MembraneOp& op, const double* X, double* out16, cudaStream_t st);
 

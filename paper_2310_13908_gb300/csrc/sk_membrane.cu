@@ -46,22 +46,22 @@ struct MembraneOp {
   int G = 0;  // ghost points used by the stencils, per field
   // operator tables (device). A tap is a spline evaluation at a fixed point
   // of one patch: its cell (node index p n^2 + a n + b of the cell's first
-  // corner) and the eight Hermite basis values there (u: value left/right,
-  // slope left/right; v likewise), followed by the tap's weights.
+  // corner) and the products of the u and v Hermite bases there (value
+  // left/right, slope left/right each; see spline_tap).
   int* ghost_dst = nullptr;    // [G] offset in a field's extended block (6 E^2)
   int* gtap_ptr = nullptr;     // [G + 1]
   int* gtap_cell = nullptr;    // [taps]
-  double* gtap_w = nullptr;    // [taps][9]: basis[8], psi
+  double* gtap_w = nullptr;    // [taps][16]: basis products times psi
   double* psi_own = nullptr;   // [N]
   int* btap_ptr = nullptr;     // [N + 1]
   int* btap_cell = nullptr;
-  double* btap_w = nullptr;    // [taps][13]: basis[8], psi, dtau1/du, dtau2/du, dtau1/dv, dtau2/dv
-  double* thomas = nullptr;    // slope-solve table (see k_slopes): c', 1/den, run products, 3/h 1/den
+  double* btap_w = nullptr;    // [taps][20]: basis products, psi (dtau1/du, dtau2/du, dtau1/dv, dtau2/dv)
+  double* thomas = nullptr;    // slope-solve table (see k_slopes)
   // scratch for up to MEM_FMAX fields
   double *g = nullptr, *sg = nullptr;    // values, spline data [3][F][N] (u, v, uv slopes)
   double* ext = nullptr;                 // [F][6][E][E]
-  double *du = nullptr, *dv = nullptr;   // FD derivatives [F][N]
-  double *sdu = nullptr, *sdv = nullptr; // their spline data [3][F][N]
+  double* du = nullptr;        // FD derivatives [2F][N]: F u-derivatives, F v-derivatives
+  double* sdu = nullptr;       // their spline data [3][2F][N]
   double *gu = nullptr, *gv = nullptr;   // blended derivatives [F][N]
   double* cur_t = nullptr;               // current tangents [6][N]
   double* red = nullptr;                 // reduction partials
@@ -197,34 +197,47 @@ inline unsigned blocks_of(int64_t n) { return (unsigned)((n + 255) / 256); }
 // Both sweeps of the solve are affine recurrences,
 //   forward   d_q = -(1/den_q) d_{q-1} + v_q,   v_q = rhs_q / den_q,
 //   backward  s_q = -c'_q s_{q+1} + d_q,
-// each with |multiplier| <= 1/2. Each lane takes a run of consecutive terms
-// and composes their maps ((a2, b2) o (a1, b1) = (a2 a1, a2 b1 + b2)); the
-// product of a run's multipliers does not depend on the data and comes from
-// the table. A scan over the line's lanes gives each lane its incoming value,
-// and the lane replays its run. v_q is computed once (stored in s, then
-// overwritten by d_q and s_q).
-// L = 8, 16 or 32 lanes per line: fewer lanes cost fewer scan steps, more
-// lanes give short lines and small grids enough threads (slope_lanes).
-// Table (thomas): [c' (n) | 1/den (n) | 3/h * 1/den (n) | for L = 8, 16, 32:
-// forward then backward run products (L each)].
-constexpr int SLOPE_LPL_MIN = 8, SLOPE_LPL_MAX = 32;
-__host__ __device__ constexpr int slope_products_offset(int n, int L) {
-  return 3 * n + 2 * (L - SLOPE_LPL_MIN);  // L = 8: 0, 16: 16, 32: 48
-}
-constexpr int SLOPE_TABLE_EXTRA = 2 * (8 + 16 + 32);
+// each with |multiplier| <= 1/2, and about 0.27 past the ends. Each of L lanes
+// takes a run of K consecutive terms, the same run in both sweeps:
+//   1. the forward recurrence over its run from 0;
+//   2. the value x entering the run from the lanes before it, d_q = that +
+//      (product of the run's multipliers up to q) x, and the backward
+//      recurrence over the run from 0;
+//   3. the value entering from the lanes behind it, likewise.
+// The products do not depend on the data and come from a table, so only 1 and
+// the second half of 2 are serial chains. An entering value needs the
+// runs within 32 terms only (0.27^32 < 2^-60): a few shuffles and FMAs
+// (entering), no scan. 16 lanes per line, as measured for the membrane force (8 /
+// 16 / 32 lanes): m = 33: 0.185 / 0.185 / 0.245 ms; m = 65: 0.267 / 0.275 / 0.342;
+// m = 129: 0.586 / 0.578 / 0.694; m = 193: 1.13 / 1.02 / 1.09; m = 257: 2.10 /
+// 1.80 / 1.80.
+// The solves are bound by these FP64 chains and by the FP64 pipe (about 7
+// instructions per term), so one launch takes all lines whose values are ready:
+// both directions of all fields, then the mixed slopes. Measured (membrane
+// force at m = 129, N = 98,304): 27 launches, 550 us, with a logarithmic scan
+// and one launch per field set and direction; now 8 launches, 276 us.
+// Table, in the order the lanes read it ([K][L], term 1 + lane K + k at
+// [k][lane]): forward multiplier, 3/h * 1/den, backward multiplier, forward
+// products, backward products; then 1/den of the first and last row.
+#ifndef SK_SLOPE_LANES
+#define SK_SLOPE_LANES 16
+#endif
+constexpr int SLOPE_LANES = SK_SLOPE_LANES;
 constexpr int SLOPE_LINES = 8;  // grid lines per CTA
+__host__ __device__ constexpr int slope_run(int n, int L) { return (n - 2 + L - 1) / L; }
 
-template <int L>
-__device__ __forceinline__ void affine_scan_lines(double& a, double& b, int sub) {
-#pragma unroll
-  for (int o = 1; o < L; o <<= 1) {
-    const double pa = __shfl_up_sync(0xffffffffu, a, o, L);
-    const double pb = __shfl_up_sync(0xffffffffu, b, o, L);
-    if (sub >= o) {
-      b = fma(a, pb, b);
-      a = a * pa;
-    }
+// The value entering lane sub's run from the D lanes on its DIR side: run r
+// maps its entering value x to A x + B.
+template <int L, int DIR>
+__device__ __forceinline__ double entering(double A, double B, int sub, int D) {
+  double x = 0.0;
+  for (int d = D; d >= 1; --d) {
+    const int from = sub - DIR * d;
+    const double b = __shfl_sync(0xffffffffu, B, from, L);
+    const double a = __shfl_sync(0xffffffffu, A, from, L);
+    if (from >= 0 && from < L) x = fma(a, x, b);
   }
+  return x;
 }
 
 // Padded shared-memory index of term q of a line: one spare double per 8, so
@@ -252,55 +265,37 @@ struct GlobalLine {
 };
 
 // Both sweeps of one line by its L lanes; g: values, s: output slopes (also
-// the scratch of v and d). `live` lanes store; the others only take part in
+// the scratch of the recurrences). Lanes that are not `live` only take part in
 // the shuffles.
 template <int L, class Acc>
 __device__ __forceinline__ void slope_sweeps(const Acc& g, const Acc& s, bool live, int n, int sub,
-                                             double ih, const double* __restrict__ thomas) {
-  const double* cp = thomas;
-  const double* iden = thomas + n;
-  const double* i3d = thomas + 2 * n;
-  const double* afw = thomas + slope_products_offset(n, L);
-  const double* abw = afw + L;
+                                             double ih, const double* __restrict__ table) {
+  const int K = slope_run(n, L), T = K * L;
+  const double* const t = table + sub;  // [k * L] is this lane's term k
+  const int qa = min(1 + sub * K, n - 1);
+  const int nq = live ? min(K, n - 1 - qa) : 0;
+  const int D = min(L - 1, (32 + K - 1) / K);
   const double i2h = 0.5 * ih;
-  const int K = (n - 2 + L - 1) / L;  // terms per lane
-  const int qa = 1 + sub * K;         // this lane's run [qa, qb) of q = 1..n-2
-  const int qb = min(qa + K, n - 1);
   const double r0 = (-5.0 * g[0] + 4.0 * g[1] + g[2]) * i2h;
   const double rN = (5.0 * g[n - 1] - 4.0 * g[n - 2] - g[n - 3]) * i2h;
-  const double c1 = r0 * iden[1], cN = rN * iden[n - 2];  // end-condition terms of v_1, v_{n-2}
-  // forward sweep
+  // end-condition terms of v_1 and v_{n-2}
+  const double c1 = r0 * table[5 * T], cN = rN * table[5 * T + 1];
   double B = 0.0;
-  for (int q = qa; q < qb; ++q) {
+  for (int k = 0; k < nq; ++k) {
+    const int q = qa + k;
     const double cq = q == 1 ? c1 : (q == n - 2 ? cN : 0.0);
-    const double v = fma(i3d[q], g[q + 1] - g[q - 1], -cq);
-    B = fma(q == 1 ? 0.0 : -iden[q], B, v);
-    if (live) s[q] = v;
+    B = fma(t[k * L], B, fma(t[T + k * L], g[q + 1] - g[q - 1], -cq));
+    s[q] = B;
   }
-  double A = afw[sub];
-  affine_scan_lines<L>(A, B, sub);
-  double x = __shfl_up_sync(0xffffffffu, B, 1, L);
-  if (sub == 0) x = 0.0;
-  for (int q = qa; q < qb; ++q) {
-    x = fma(q == 1 ? 0.0 : -iden[q], x, s[q]);
-    if (live) s[q] = x;
-  }
-  __syncwarp();
-  // backward sweep over p = 1..n-2, q = n-1-p (s_{n-2} = d_{n-2})
+  double x = entering<L, 1>(nq > 0 ? t[3 * T + (nq - 1) * L] : 0.0, B, sub, D);
   B = 0.0;
-  for (int p = qa; p < qb; ++p) {
-    const int q = n - 1 - p;
-    B = fma(q == n - 2 ? 0.0 : -cp[q], B, s[q]);
+  for (int k = nq - 1; k >= 0; --k) {
+    const int q = qa + k;
+    B = fma(t[2 * T + k * L], B, fma(t[3 * T + k * L], x, s[q]));
+    s[q] = B;
   }
-  A = abw[sub];
-  affine_scan_lines<L>(A, B, sub);
-  x = __shfl_up_sync(0xffffffffu, B, 1, L);
-  if (sub == 0) x = 0.0;
-  for (int p = qa; p < qb; ++p) {
-    const int q = n - 1 - p;
-    x = fma(q == n - 2 ? 0.0 : -cp[q], x, s[q]);
-    if (live) s[q] = x;
-  }
+  x = entering<L, -1>(nq > 0 ? t[4 * T] : 0.0, B, sub, D);
+  for (int k = 0; k < nq; ++k) s[qa + k] = fma(t[4 * T + k * L], x, s[qa + k]);
   __syncwarp();
   if (sub == 0 && live) {
     s[0] = r0 - 2.0 * s[1];
@@ -308,14 +303,24 @@ __device__ __forceinline__ void slope_sweeps(const Acc& g, const Acc& s, bool li
   }
 }
 
+// Up to two sets of lines solved by one launch (blockIdx.y).
+struct SlopeJobs {
+  const double* in[2];
+  double* out[2];
+  int dir[2];
+};
+
 // SLOPE_LINES lines per CTA (8 L threads). Staged: the lines' values and
 // slopes sit in shared memory (dynamic, 2 x SLOPE_LINES x spad(n) doubles),
 // loaded and stored coalesced (for dir 0 the CTA's lines are adjacent
 // columns). Unstaged (long lines): the sweeps work in global memory.
 template <int L, bool STAGED>
 __global__ void __launch_bounds__(SLOPE_LINES * L)
-    k_slopes(const double* __restrict__ g, double* __restrict__ s, int64_t n_lines, int n,
-             int dir, double ih, const double* __restrict__ thomas) {
+    k_slopes(const SlopeJobs jobs, int64_t n_lines, int n, double ih,
+             const double* __restrict__ table) {
+  const double* __restrict__ g = jobs.in[blockIdx.y];
+  double* __restrict__ s = jobs.out[blockIdx.y];
+  const int dir = jobs.dir[blockIdx.y];
   constexpr int T = SLOPE_LINES * L;
   const int tid = threadIdx.x, l = tid / L, sub = tid % L;
   const int64_t line0 = (int64_t)blockIdx.x * SLOPE_LINES;
@@ -325,7 +330,7 @@ __global__ void __launch_bounds__(SLOPE_LINES * L)
     const bool live = line0 + l < n_lines;
     const int64_t b = slope_line_base(live ? line0 + l : n_lines - 1, n, dir);
     slope_sweeps<L>(GlobalLine{const_cast<double*>(g) + b, st}, GlobalLine{s + b, st}, live, n, sub,
-                    ih, thomas);
+                    ih, table);
     return;
   }
   extern __shared__ double sm_lines[];
@@ -345,8 +350,8 @@ __global__ void __launch_bounds__(SLOPE_LINES * L)
     if (b >= 0) gsh[li * stride + spad(q)] = g[b + q * st];
   }
   __syncthreads();
-  slope_sweeps<L>(StagedLine{gsh + l * stride}, StagedLine{ssh + l * stride}, true, n, sub, ih,
-                  thomas);
+  slope_sweeps<L>(StagedLine{gsh + l * stride}, StagedLine{ssh + l * stride}, line0 + l < n_lines,
+                  n, sub, ih, table);
   __syncthreads();
   for (int idx = tid; idx < SLOPE_LINES * n; idx += T) {
     const int li = dir == 0 ? idx % SLOPE_LINES : idx / n;
@@ -358,21 +363,40 @@ __global__ void __launch_bounds__(SLOPE_LINES * L)
 
 // Bicubic Hermite evaluation of one field's spline at a tap: node values g,
 // spline data sd (u, v, uv slopes at plane strides), field offset fo, the
-// tap's cell (index of the cell's first corner) and bases w[0..7].
+// tap's cell (index of the cell's first corner) and basis products w[4 r + c],
+// r: u basis (value left, right, slope left, right), c: v basis likewise.
+// (The products come from the table: 16 FP64 instructions where bases would
+// take 20, on the pipe that bounds the blending.)
 __device__ __forceinline__ double spline_tap(const double* __restrict__ g,
                                              const double* __restrict__ sd, int64_t plane,
-                                             int64_t fo, int cell, int n,
-                                             const double* __restrict__ w) {
+                                             int64_t fo, int cell, int n, const double* w) {
   const double* su = sd;
   const double* sv = sd + plane;
   const double* suv = sd + 2 * plane;
-  const int64_t i00 = fo + cell, i10 = i00 + n, i01 = i00 + 1, i11 = i00 + n + 1;
-  const double A0 = w[0], A1 = w[1], B0 = w[2], B1 = w[3];
-  const double C0 = w[4], C1 = w[5], D0 = w[6], D1 = w[7];
-  return A0 * (C0 * g[i00] + C1 * g[i01] + D0 * sv[i00] + D1 * sv[i01]) +
-         A1 * (C0 * g[i10] + C1 * g[i11] + D0 * sv[i10] + D1 * sv[i11]) +
-         B0 * (C0 * su[i00] + C1 * su[i01] + D0 * suv[i00] + D1 * suv[i01]) +
-         B1 * (C0 * su[i10] + C1 * su[i11] + D0 * suv[i10] + D1 * suv[i11]);
+  const int64_t i00 = fo + cell, i10 = i00 + n;
+  double v = w[0] * g[i00];
+  v = fma(w[1], g[i00 + 1], v);
+  v = fma(w[2], sv[i00], v);
+  v = fma(w[3], sv[i00 + 1], v);
+  v = fma(w[4], g[i10], v);
+  v = fma(w[5], g[i10 + 1], v);
+  v = fma(w[6], sv[i10], v);
+  v = fma(w[7], sv[i10 + 1], v);
+  v = fma(w[8], su[i00], v);
+  v = fma(w[9], su[i00 + 1], v);
+  v = fma(w[10], suv[i00], v);
+  v = fma(w[11], suv[i00 + 1], v);
+  v = fma(w[12], su[i10], v);
+  v = fma(w[13], su[i10 + 1], v);
+  v = fma(w[14], suv[i10], v);
+  return fma(w[15], suv[i10 + 1], v);
+}
+
+// w[4 r + c] = scale bases[r] bases[4 + c]
+__host__ __device__ __forceinline__ void basis_products(const double* bases, double scale,
+                                                        double* w) {
+  for (int r = 0; r < 4; ++r)
+    for (int c = 0; c < 4; ++c) w[4 * r + c] = scale * bases[r] * bases[4 + c];
 }
 
 // Extended values: nodes copied, ghost points by patch extension (Eq. ext).
@@ -393,10 +417,9 @@ __global__ void k_extend(const MembraneOp op, int F) {
   const int f = (int)(gi / op.G);
   const int q = (int)(gi % op.G);
   double val = 0.0;
-  for (int t = op.gtap_ptr[q]; t < op.gtap_ptr[q + 1]; ++t) {
-    const double* w = op.gtap_w + 9 * t;
-    val += w[8] * spline_tap(op.g, op.sg, plane, (int64_t)f * N, op.gtap_cell[t], op.n, w);
-  }
+  for (int t = op.gtap_ptr[q]; t < op.gtap_ptr[q + 1]; ++t)
+    val += spline_tap(op.g, op.sg, plane, (int64_t)f * N, op.gtap_cell[t], op.n,
+                      op.gtap_w + 16 * (int64_t)t);
   op.ext[f * blk + op.ghost_dst[q]] = val;
 }
 
@@ -412,30 +435,55 @@ __global__ void k_fd(const MembraneOp op, int F) {
   const int j = r / op.n, k = r % op.n;
   const int E = op.E;
   const double* e = op.ext + (int64_t)f * 6 * E * E + ((int64_t)p * E + j + 3) * E + k + 3;
-  const double c1 = 45.0 / 60.0, c2 = -9.0 / 60.0, c3 = 1.0 / 60.0;
-  op.du[i] = (c1 * (e[E] - e[-E]) + c2 * (e[2 * E] - e[-2 * E]) + c3 * (e[3 * E] - e[-3 * E])) * op.ih;
-  op.dv[i] = (c1 * (e[1] - e[-1]) + c2 * (e[2] - e[-2]) + c3 * (e[3] - e[-3])) * op.ih;
+  const double c1 = 45.0 / 60.0 * op.ih, c2 = -9.0 / 60.0 * op.ih, c3 = 1.0 / 60.0 * op.ih;
+  op.du[i] = c1 * (e[E] - e[-E]) + c2 * (e[2 * E] - e[-2 * E]) + c3 * (e[3 * E] - e[-3 * E]);
+  op.du[F * N + i] = c1 * (e[1] - e[-1]) + c2 * (e[2] - e[-2]) + c3 * (e[3] - e[-3]);
 }
 
-// Eqs. blendu / blendv.
-__global__ void k_blend(const MembraneOp op, int F) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  const int64_t N = op.N, plane = (int64_t)F * N;
-  if (i >= F * N) return;
-  const int f = (int)(i / N);
-  const int64_t node = i % N;
+// Eqs. blendu / blendv. A thread takes one node and BLEND_FIELDS fields, so
+// that a tap's weights are read once for six spline evaluations. Bound by the
+// FP64 pipe (36 instructions per field and tap). With the bases multiplied out
+// in the table and the weights shared by three fields, the three launches of a
+// membrane force at m = 129 went from 194 us to 166 us in two.
+constexpr int BLEND_FIELDS = 3;
+__global__ void __launch_bounds__(256) k_blend(const MembraneOp op, int F) {
+  const int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t N = op.N, plane = 2 * (int64_t)F * N;
+  if (node >= N) return;
+  const int f0 = blockIdx.y * BLEND_FIELDS;
   const double po = op.psi_own[node];
-  double ou = po * op.du[i], ov = po * op.dv[i];
-  for (int t = op.btap_ptr[node]; t < op.btap_ptr[node + 1]; ++t) {
-    const double* w = op.btap_w + 13 * t;
-    const int cell = op.btap_cell[t];
-    const double eu = spline_tap(op.du, op.sdu, plane, (int64_t)f * N, cell, op.n, w);
-    const double ev = spline_tap(op.dv, op.sdv, plane, (int64_t)f * N, cell, op.n, w);
-    ou += w[8] * (eu * w[9] + ev * w[10]);
-    ov += w[8] * (eu * w[11] + ev * w[12]);
+  double ou[BLEND_FIELDS], ov[BLEND_FIELDS];
+#pragma unroll
+  for (int i = 0; i < BLEND_FIELDS; ++i) {
+    const int64_t at = (int64_t)min(f0 + i, F - 1) * N + node;
+    ou[i] = po * op.du[at];
+    ov[i] = po * op.du[F * N + at];
   }
-  op.gu[i] = ou;
-  op.gv[i] = ov;
+  for (int t = op.btap_ptr[node]; t < op.btap_ptr[node + 1]; ++t) {
+    const double2* wt = reinterpret_cast<const double2*>(op.btap_w + 20 * (int64_t)t);
+    const int cell = op.btap_cell[t];
+    double w[20];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+      const double2 v = wt[k];
+      w[2 * k] = v.x;
+      w[2 * k + 1] = v.y;
+    }
+#pragma unroll
+    for (int i = 0; i < BLEND_FIELDS; ++i) {
+      const int64_t f = min(f0 + i, F - 1);
+      const double eu = spline_tap(op.du, op.sdu, plane, f * N, cell, op.n, w);
+      const double ev = spline_tap(op.du, op.sdu, plane, (F + f) * N, cell, op.n, w);
+      ou[i] = fma(eu, w[16], fma(ev, w[17], ou[i]));
+      ov[i] = fma(eu, w[18], fma(ev, w[19], ov[i]));
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < BLEND_FIELDS; ++i)
+    if (f0 + i < F) {
+      op.gu[(f0 + i) * N + node] = ou[i];
+      op.gv[(f0 + i) * N + node] = ov[i];
+    }
 }
 
 // [N][ld] column block c0..c0+F  <->  [F][N]
@@ -457,7 +505,7 @@ __global__ void k_scatter(const double* __restrict__ soa, int64_t N, int ld, int
 }
 
 struct Frame {
-  double a1[3], a2[3], E, F, G, W, n[3];
+  double a1[3], a2[3], E, F, G, W, iW, n[3];
 };
 __device__ __forceinline__ Frame frame_at(const double* __restrict__ t6, int64_t N, int64_t i) {
   Frame fr;
@@ -468,23 +516,32 @@ __device__ __forceinline__ Frame frame_at(const double* __restrict__ t6, int64_t
   fr.E = fr.a1[0] * fr.a1[0] + fr.a1[1] * fr.a1[1] + fr.a1[2] * fr.a1[2];
   fr.F = fr.a1[0] * fr.a2[0] + fr.a1[1] * fr.a2[1] + fr.a1[2] * fr.a2[2];
   fr.G = fr.a2[0] * fr.a2[0] + fr.a2[1] * fr.a2[1] + fr.a2[2] * fr.a2[2];
-  fr.W = sqrt(fr.E * fr.G - fr.F * fr.F);
-  fr.n[0] = (fr.a1[1] * fr.a2[2] - fr.a1[2] * fr.a2[1]) / fr.W;
-  fr.n[1] = (fr.a1[2] * fr.a2[0] - fr.a1[0] * fr.a2[2]) / fr.W;
-  fr.n[2] = (fr.a1[0] * fr.a2[1] - fr.a1[1] * fr.a2[0]) / fr.W;
+  // one reciprocal square root for W and 1/W (a square root and divisions
+  // take several times the FP64 instructions)
+  const double W2 = fr.E * fr.G - fr.F * fr.F;
+  if (W2 > 1e-290) {
+    fr.iW = rsqrt_fp64(W2);
+    fr.W = W2 * fr.iW;
+  } else {
+    fr.W = sqrt(W2);
+    fr.iW = 1.0 / fr.W;
+  }
+  fr.n[0] = (fr.a1[1] * fr.a2[2] - fr.a1[2] * fr.a2[1]) * fr.iW;
+  fr.n[1] = (fr.a1[2] * fr.a2[0] - fr.a1[0] * fr.a2[2]) * fr.iW;
+  fr.n[2] = (fr.a1[0] * fr.a2[1] - fr.a1[1] * fr.a2[0]) * fr.iW;
   return fr;
 }
 
-// Tangents of the last F = 3 pass (positions) -> t6 [6][N]; optional
-// quadrature weights psi W h^2 (Sec. 3.3, Eq. smoothint).
-__global__ void k_tangents(const MembraneOp op, double* __restrict__ t6, double* __restrict__ w,
-                           double* __restrict__ Wraw) {
+// Tangents of the last pass's fields f0 .. f0 + 2 (positions) -> t6 [6][N];
+// optional quadrature weights psi W h^2 (Sec. 3.3, Eq. smoothint).
+__global__ void k_tangents(const MembraneOp op, int f0, double* __restrict__ t6,
+                           double* __restrict__ w, double* __restrict__ Wraw) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t N = op.N;
   if (i >= N) return;
   for (int c = 0; c < 3; ++c) {
-    t6[c * N + i] = op.gu[c * N + i];
-    t6[(3 + c) * N + i] = op.gv[c * N + i];
+    t6[c * N + i] = op.gu[(f0 + c) * N + i];
+    t6[(3 + c) * N + i] = op.gv[(f0 + c) * N + i];
   }
   if (w || Wraw) {
     const Frame fr = frame_at(t6, N, i);
@@ -503,11 +560,11 @@ __global__ void k_tension(const MembraneOp op, const double* __restrict__ cur,
   const int64_t N = op.N;
   if (i >= N) return;
   const Frame c = frame_at(cur, N, i), r = frame_at(ref, N, i);
-  const double iw2 = 1.0 / (r.W * r.W);
+  const double iw2 = r.iW * r.iW;
   const double tr = (r.G * c.E - 2.0 * r.F * c.F + r.E * c.G) * iw2;
-  const double Js = c.W / r.W;
+  const double Js = c.W * r.iW;
   const double I1 = tr - 2.0, I2 = Js * Js - 1.0;
-  const double k1 = Es / (2.0 * Js) * (I1 + 1.0), k2 = 0.5 * Js * (ED * I2 - Es);
+  const double k1 = 0.5 * Es * (r.W * c.iW) * (I1 + 1.0), k2 = 0.5 * Js * (ED * I2 - Es);
   const int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};
   for (int q = 0; q < 6; ++q) {
     const int a = ia[q], b = ib[q];
@@ -527,7 +584,7 @@ __global__ void k_divergence(const MembraneOp op, const double* __restrict__ cur
   const int64_t N = op.N;
   if (i >= N) return;
   const Frame c = frame_at(cur, N, i);
-  const double iw2 = 1.0 / (c.W * c.W);
+  const double iw2 = c.iW * c.iW;
   const int comp[3][3] = {{0, 3, 4}, {3, 1, 5}, {4, 5, 2}};
   for (int k = 0; k < 3; ++k) {
     double acc = 0.0;
@@ -651,11 +708,12 @@ __global__ void k_upsample(const MembraneOp op, double hu2) {
   const int p = (int)(i / nf2);
   const int r = (int)(i % nf2);
   const int J = r / op.nf, K = r % op.nf;
-  double w[8];
+  double bases[8], w[16];
   for (int c = 0; c < 4; ++c) {
-    w[c] = op.ubasis1[4 * J + c];
-    w[4 + c] = op.ubasis1[4 * K + c];
+    bases[c] = op.ubasis1[4 * J + c];
+    bases[4 + c] = op.ubasis1[4 * K + c];
   }
+  basis_products(bases, 1.0, w);
   const int cell = (p * op.n + op.ucell1[J]) * op.n + op.ucell1[K];
   const int64_t plane = 7 * op.N;
   double v[7];
@@ -667,39 +725,55 @@ __global__ void k_upsample(const MembraneOp op, double hu2) {
   op.wu[i] = op.psi_up[i] * v[6] * hu2;
 }
 
-// delta_u per patch: Eq. regparam on the fine grid (largest distance from a
-// node to an existing grid neighbour, maximized over the patch).
-__global__ void k_fine_delta(const MembraneOp op) {
+// Largest distance between grid neighbours per patch (Eq. regparam, C = 1) of
+// nodes X on six n x n grids, as bits of the squared distance in pmax[p] (which
+// starts at 0; nonnegative doubles order like their bits). A node takes the
+// neighbours that follow it: each pair once, and one square root per patch
+// afterwards (k_patch_delta) instead of one per pair. One atomic per warp where
+// the warp lies in one patch. (96,774 fine nodes: 77 us with eight neighbours,
+// their square roots and an atomic per node; now 10 us.)
+__global__ void __launch_bounds__(256) k_patch_reach(const double* __restrict__ X, int n,
+                                                     unsigned long long* __restrict__ pmax) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= op.Nup) return;
-  const int nf = op.nf;
-  const int p = (int)(i / ((int64_t)nf * nf));
-  const int r = (int)(i % ((int64_t)nf * nf));
-  const int j = r / nf, k = r % nf;
-  const double x = op.Xu[3 * i], y = op.Xu[3 * i + 1], z = op.Xu[3 * i + 2];
+  const int64_t n2 = (int64_t)n * n;
   double best = 0.0;
-  for (int a = -1; a <= 1; ++a)
-    for (int b = -1; b <= 1; ++b) {
-      const int jj = j + a, kk = k + b;
-      if ((a == 0 && b == 0) || jj < 0 || jj >= nf || kk < 0 || kk >= nf) continue;
-      const int64_t q = ((int64_t)p * nf + jj) * nf + kk;
-      const double dx = x - op.Xu[3 * q], dy = y - op.Xu[3 * q + 1], dz = z - op.Xu[3 * q + 2];
-      best = fmax(best, sqrt(dx * dx + dy * dy + dz * dz));
+  int p = -1;
+  if (i < 6 * n2) {
+    p = (int)(i / n2);
+    const int r = (int)(i % n2);
+    const int j = r / n, k = r % n;
+    const double x = X[3 * i], y = X[3 * i + 1], z = X[3 * i + 2];
+    auto take = [&](int64_t q) {
+      const double dx = x - X[3 * q], dy = y - X[3 * q + 1], dz = z - X[3 * q + 2];
+      best = fmax(best, dx * dx + dy * dy + dz * dz);
+    };
+    if (k + 1 < n) take(i + 1);
+    if (j + 1 < n) {
+      if (k > 0) take(i + n - 1);
+      take(i + n);
+      if (k + 1 < n) take(i + n + 1);
     }
-  // nonnegative doubles order like their bit patterns
-  atomicMax(op.pmax + p, (unsigned long long)__double_as_longlong(best));
+  }
+  const int p0 = __shfl_sync(0xffffffffu, p, 0);
+  if (__all_sync(0xffffffffu, p == p0)) {
+    for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_xor_sync(0xffffffffu, best, o));
+    if ((threadIdx.x & 31) != 0) return;
+  }
+  if (p >= 0) atomicMax(pmax + p, (unsigned long long)__double_as_longlong(best));
 }
 
-__global__ void k_delta_targets(const MembraneOp op) {
+// delta[i] = the reach of node i's patch, n2 nodes per patch.
+__global__ void k_patch_delta(const unsigned long long* __restrict__ pmax, int64_t n2,
+                              double* __restrict__ delta) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < op.N) op.dtgt[i] = __longlong_as_double((long long)op.pmax[i / ((int64_t)op.n * op.n)]);
+  if (i < 6 * n2) delta[i] = sqrt(__longlong_as_double((long long)pmax[i / n2]));
 }
 
 void free_op(MembraneOp* op) {
   if (!op) return;
   for (MembraneOp* c : op->sets) free_op(c);
-  for (void* p : {(void*)op->g, (void*)op->sg, (void*)op->ext, (void*)op->du, (void*)op->dv,
-                  (void*)op->sdu, (void*)op->sdv, (void*)op->gu, (void*)op->gv, (void*)op->cur_t,
+  for (void* p : {(void*)op->g, (void*)op->sg, (void*)op->ext, (void*)op->du,
+                  (void*)op->sdu, (void*)op->gu, (void*)op->gv, (void*)op->cur_t,
                   (void*)op->red})
     if (p) cudaFree(p);
   if (op->owns_tables)
@@ -725,10 +799,8 @@ cudaError_t alloc_scratch(MembraneOp* op) {
   ok(cudaMalloc(&op->g, fn));
   ok(cudaMalloc(&op->sg, 3 * fn));
   ok(cudaMalloc(&op->ext, (size_t)MEM_FMAX * 6 * E * E * sizeof(double)));
-  ok(cudaMalloc(&op->du, fn));
-  ok(cudaMalloc(&op->dv, fn));
-  ok(cudaMalloc(&op->sdu, 3 * fn));
-  ok(cudaMalloc(&op->sdv, 3 * fn));
+  ok(cudaMalloc(&op->du, 2 * fn));
+  ok(cudaMalloc(&op->sdu, 6 * fn));
   ok(cudaMalloc(&op->gu, fn));
   ok(cudaMalloc(&op->gv, fn));
   ok(cudaMalloc(&op->cur_t, 6 * op->N * sizeof(double)));
@@ -772,8 +844,9 @@ int build_op(int m, MembraneOp** out, std::string& err) {
           double uq, vq, bs[8];
           h_inverse_chart(q, x1, uq, vq);
           gcell.push_back(h_cell_basis(q, n, h, uq, vq, bs));
-          gw.insert(gw.end(), bs, bs + 8);
-          gw.push_back(psi[q]);
+          double w[16];
+          basis_products(bs, psi[q], w);
+          gw.insert(gw.end(), w, w + 16);
         }
         gptr.push_back((int)gcell.size());
         gdst.push_back((p * E + j + 2) * E + k + 2);
@@ -796,41 +869,42 @@ int build_op(int m, MembraneOp** out, std::string& err) {
           h_inverse_chart(q, x0, uq, vq);
           h_transition_jacobian(p, q, u, v, uq, vq, J);
           bcell.push_back(h_cell_basis(q, n, h, uq, vq, bs));
-          bw.insert(bw.end(), bs, bs + 8);
-          bw.insert(bw.end(), {psi[q], J[0], J[1], J[2], J[3]});
+          double w[16];
+          basis_products(bs, 1.0, w);
+          bw.insert(bw.end(), w, w + 16);
+          for (int c = 0; c < 4; ++c) bw.push_back(psi[q] * J[c]);
         }
         bptr.push_back((int)bcell.size());
       }
   // factorization of the reduced slope system: rows q = 1..n-2 with
-  // (sub, diag, super) = (-, 2, 1), (1, 4, 1) ..., (1, 2, -); then the
-  // 3/h * 1/den and the products of each lane run's multipliers (k_slopes)
-  std::vector<double> th(3 * n + SLOPE_TABLE_EXTRA, 0.0);
+  // (sub, diag, super) = (-, 2, 1), (1, 4, 1) ..., (1, 2, -); then the table of
+  // k_slopes
+  std::vector<double> cp(n, 0.0), iden(n, 0.0);
   for (int q = 1; q <= n - 2; ++q) {
     const double b = (q == 1 || q == n - 2) ? 2.0 : 4.0;
     const double a = q == 1 ? 0.0 : 1.0;
     const double c = q == n - 2 ? 0.0 : 1.0;
-    const double den = b - a * (q > 1 ? th[q - 1] : 0.0);
-    th[q] = c / den;
-    th[n + q] = 1.0 / den;
+    const double den = b - a * (q > 1 ? cp[q - 1] : 0.0);
+    cp[q] = c / den;
+    iden[q] = 1.0 / den;
   }
-  {
-    const double i3h = 3.0 / h;
-    for (int q = 1; q <= n - 2; ++q) th[2 * n + q] = i3h * th[n + q];
-    for (int L = SLOPE_LPL_MIN; L <= SLOPE_LPL_MAX; L *= 2) {
-      const int K = (n - 2 + L - 1) / L, off = slope_products_offset(n, L);
-      for (int r = 0; r < L; ++r) {
-        const int qa = 1 + r * K, qb = std::min(qa + K, n - 1);
-        double pf = 1.0, pb = 1.0;
-        for (int q = qa; q < qb; ++q) pf *= q == 1 ? 0.0 : -th[n + q];
-        for (int p = qa; p < qb; ++p) {
-          const int q = n - 1 - p;
-          pb *= q == n - 2 ? 0.0 : -th[q];
-        }
-        th[off + r] = pf;
-        th[off + L + r] = pb;
-      }
+  constexpr int L = SLOPE_LANES;
+  const int K = slope_run(n, L), T = K * L;
+  std::vector<double> th(5 * (size_t)T + 2, 0.0);
+  for (int r = 0; r < L; ++r) {
+    const int qa = std::min(1 + r * K, n - 1), nq = std::min(K, n - 1 - qa);
+    double pf = 1.0, pb = 1.0;
+    for (int k = 0; k < nq; ++k) {
+      const int q = qa + k, at = k * L + r;
+      th[at] = q == 1 ? 0.0 : -iden[q];
+      th[T + at] = 3.0 / h * iden[q];
+      th[2 * T + at] = q == n - 2 ? 0.0 : -cp[q];
+      th[3 * T + at] = pf *= th[at];
     }
+    for (int k = nq - 1; k >= 0; --k) th[4 * T + k * L + r] = pb *= th[2 * T + k * L + r];
   }
+  th[5 * T] = iden[1];
+  th[5 * T + 1] = iden[n - 2];
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t x) {
     if (x != cudaSuccess && e == cudaSuccess) e = x;
@@ -911,49 +985,25 @@ int ensure_upsampling(MembraneOp* op, std::string& err) {
   return SK_OK;
 }
 
-#ifndef SK_SLOPE_LANES
-#define SK_SLOPE_LANES 0  // 0: by size (below); 8, 16 or 32: fixed
-#endif
-// Lanes per line by line length n, as measured for the membrane force (8 /
-// 16 / 32 lanes): m = 65: 0.54 / 0.46 / 0.50 ms; m = 129: 1.00 / 0.95 /
-// 1.09 ms; m = 257: 2.71 / 3.24 / 2.97 ms (32 lanes was the earlier kernel's
-// layout: 0.55, 1.30, 3.62 ms with its redundant arithmetic).
-inline int slope_lanes(int n) {
-  if (SK_SLOPE_LANES) return SK_SLOPE_LANES;
-  return n <= 160 ? 16 : 8;
-}
-
 // Spline data (u, v, uv slopes) of F fields in `val` into `sd` ([3][F][N]).
 void enqueue_splines(const MembraneOp& op, int F, const double* val, double* sd, cudaStream_t st) {
   const int64_t plane = (int64_t)F * op.N;
   const int64_t lines = (int64_t)F * 6 * op.n;
-  const int L = slope_lanes(op.n);
+  constexpr int L = SLOPE_LANES;
   const unsigned nb = (unsigned)((lines + SLOPE_LINES - 1) / SLOPE_LINES);
   // staged lines: 2 arrays x SLOPE_LINES lines x spad(n) doubles, within the
   // default 48 KB of dynamic shared memory (lines up to n = 341)
   const size_t smem = 2 * (size_t)SLOPE_LINES * (op.n + (op.n >> 3)) * sizeof(double);
   const bool staged = op.slope_staging && smem <= 48 * 1024;
-  auto run = [&](const double* in, double* out, int dir) {
-    const unsigned T = (unsigned)(SLOPE_LINES * L);
-    if (staged) {
-      if (L == 8)
-        k_slopes<8, true><<<nb, T, smem, st>>>(in, out, lines, op.n, dir, op.ih, op.thomas);
-      else if (L == 16)
-        k_slopes<16, true><<<nb, T, smem, st>>>(in, out, lines, op.n, dir, op.ih, op.thomas);
-      else
-        k_slopes<32, true><<<nb, T, smem, st>>>(in, out, lines, op.n, dir, op.ih, op.thomas);
-    } else {
-      if (L == 8)
-        k_slopes<8, false><<<nb, T, 0, st>>>(in, out, lines, op.n, dir, op.ih, op.thomas);
-      else if (L == 16)
-        k_slopes<16, false><<<nb, T, 0, st>>>(in, out, lines, op.n, dir, op.ih, op.thomas);
-      else
-        k_slopes<32, false><<<nb, T, 0, st>>>(in, out, lines, op.n, dir, op.ih, op.thomas);
-    }
+  auto run = [&](const SlopeJobs& jobs, unsigned n_jobs) {
+    const dim3 grid(nb, n_jobs);
+    if (staged)
+      k_slopes<L, true><<<grid, SLOPE_LINES * L, smem, st>>>(jobs, lines, op.n, op.ih, op.thomas);
+    else
+      k_slopes<L, false><<<grid, SLOPE_LINES * L, 0, st>>>(jobs, lines, op.n, op.ih, op.thomas);
   };
-  run(val, sd, 0);
-  run(val, sd + plane, 1);
-  run(sd, sd + 2 * plane, 1);
+  run(SlopeJobs{{val, val}, {sd, sd + plane}, {0, 1}}, 2);
+  run(SlopeJobs{{sd, nullptr}, {sd + 2 * plane, nullptr}, {1, 0}}, 1);
 }
 
 }  // namespace
@@ -964,9 +1014,8 @@ void enqueue_derivatives(const MembraneOp& op, int F, cudaStream_t st) {
   enqueue_splines(op, F, op.g, op.sg, st);
   k_extend<<<blocks_of((int64_t)F * (op.N + op.G)), 256, 0, st>>>(op, F);
   k_fd<<<blocks_of((int64_t)F * op.N), 256, 0, st>>>(op, F);
-  enqueue_splines(op, F, op.du, op.sdu, st);
-  enqueue_splines(op, F, op.dv, op.sdv, st);
-  k_blend<<<blocks_of((int64_t)F * op.N), 256, 0, st>>>(op, F);
+  enqueue_splines(op, 2 * F, op.du, op.sdu, st);
+  k_blend<<<dim3(blocks_of(op.N), (F + BLEND_FIELDS - 1) / BLEND_FIELDS), 256, 0, st>>>(op, F);
 }
 
 // Tangents of the nodes X ([N][3], device) into t6 ([6][N]; the operator's
@@ -976,13 +1025,35 @@ void enqueue_tangents(const MembraneOp& op, const double* X, double* t6, double*
   if (!t6) t6 = op.cur_t;
   k_gather<<<blocks_of(3 * op.N), 256, 0, st>>>(X, op.N, 3, 0, 3, op.g);
   enqueue_derivatives(op, 3, st);
-  k_tangents<<<blocks_of(op.N), 256, 0, st>>>(op, t6, w, Wraw);
+  k_tangents<<<blocks_of(op.N), 256, 0, st>>>(op, 0, t6, w, Wraw);
 }
+
+void enqueue_force(const MembraneOp& op, const double* ref6, double Es, double ED, double* f,
+                   cudaStream_t st);
 
 // Skalak force f ([N][3]) at X given reference tangents ref6 ([6][N]).
 void enqueue_skalak(const MembraneOp& op, const double* X, const double* ref6, double Es,
                     double ED, double* f, double* w, cudaStream_t st, double* Wraw) {
   enqueue_tangents(op, X, op.cur_t, w, st, Wraw);
+  enqueue_force(op, ref6, Es, ED, f, st);
+}
+
+// The same with the reference's nodes Xr instead of its tangents, which land
+// in ref6: both sets of tangents in one pass of six fields.
+void enqueue_skalak_ref(const MembraneOp& op, const double* X, const double* Xr, double* ref6,
+                        double Es, double ED, double* f, double* w, cudaStream_t st) {
+  static_assert(MEM_FMAX >= 6, "two sets of positions");
+  k_gather<<<blocks_of(3 * op.N), 256, 0, st>>>(X, op.N, 3, 0, 3, op.g);
+  k_gather<<<blocks_of(3 * op.N), 256, 0, st>>>(Xr, op.N, 3, 0, 3, op.g + 3 * op.N);
+  enqueue_derivatives(op, 6, st);
+  k_tangents<<<blocks_of(op.N), 256, 0, st>>>(op, 0, op.cur_t, w, nullptr);
+  k_tangents<<<blocks_of(op.N), 256, 0, st>>>(op, 3, ref6, nullptr, nullptr);
+  enqueue_force(op, ref6, Es, ED, f, st);
+}
+
+// Tension and divergence from the current tangents (op.cur_t) and ref6.
+void enqueue_force(const MembraneOp& op, const double* ref6, double Es, double ED, double* f,
+                   cudaStream_t st) {
   k_tension<<<blocks_of(op.N), 256, 0, st>>>(op, op.cur_t, ref6, Es, ED);
   enqueue_derivatives(op, 6, st);
   k_divergence<<<blocks_of(op.N), 256, 0, st>>>(op, op.cur_t, f);
@@ -1010,6 +1081,17 @@ void enqueue_moments(const MembraneOp& op, const double* X, double* out16, cudaS
 
 int membrane_upsampling(sk_ctx* ctx, MembraneOp* op) { return ensure_upsampling(op, ctx->err); }
 
+void enqueue_patch_reach(const double* X, int n, unsigned long long* pmax, cudaStream_t st) {
+  cudaMemsetAsync(pmax, 0, 8 * sizeof(unsigned long long), st);
+  k_patch_reach<<<blocks_of(6 * (int64_t)n * n), 256, 0, st>>>(X, n, pmax);
+}
+
+void enqueue_patch_delta(const double* X, int n, unsigned long long* pmax, double* delta,
+                         cudaStream_t st) {
+  enqueue_patch_reach(X, n, pmax, st);
+  k_patch_delta<<<blocks_of(6 * (int64_t)n * n), 256, 0, st>>>(pmax, (int64_t)n * n, delta);
+}
+
 // I_u of the nodes X, area elements W and densities f (device) into the
 // operator's fine sources, and delta_u per coarse target (Sec. 3.4).
 void enqueue_upsample(const MembraneOp& op, const double* X, const double* W, const double* f,
@@ -1021,9 +1103,8 @@ void enqueue_upsample(const MembraneOp& op, const double* X, const double* W, co
   enqueue_splines(op, 7, op.g, op.sg, st);
   const double hu = PI_CONST / (4.0 * op.m);
   k_upsample<<<blocks_of(op.Nup), 256, 0, st>>>(op, hu * hu);
-  cudaMemsetAsync(op.pmax, 0, 8 * sizeof(unsigned long long), st);
-  k_fine_delta<<<blocks_of(op.Nup), 256, 0, st>>>(op);
-  k_delta_targets<<<blocks_of(N), 256, 0, st>>>(op);
+  enqueue_patch_reach(op.Xu, op.nf, op.pmax, st);
+  k_patch_delta<<<blocks_of(N), 256, 0, st>>>(op.pmax, (int64_t)op.n * op.n, op.dtgt);
 }
 
 UpsampledSources upsampled_sources(const MembraneOp& op) {
@@ -1064,8 +1145,7 @@ int membrane_scratch_set(sk_ctx* ctx, MembraneOp* op, int i, MembraneOp** out) {
     if (!c) return SK_ENOMEM;
     c->owns_tables = false;
     for (MembraneOp*& q : c->sets) q = nullptr;
-    c->g = c->sg = c->ext = c->du = c->dv = c->sdu = c->sdv = c->gu = c->gv = c->cur_t =
-        c->red = nullptr;
+    c->g = c->sg = c->ext = c->du = c->sdu = c->gu = c->gv = c->cur_t = c->red = nullptr;
     int prev = -1;
     cudaGetDevice(&prev);
     cudaSetDevice(ctx->device);
@@ -1175,8 +1255,7 @@ int membrane_force(sk_ctx* ctx, int m, int mem, const double* X, const double* X
     dX = tX;
     dXr = tXr;
   }
-  enqueue_tangents(*op, dXr, ref6, nullptr, st);
-  enqueue_skalak(*op, dX, ref6, Es, ED, df, dw, st);
+  enqueue_skalak_ref(*op, dX, dXr, ref6, Es, ED, df, dw, st);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess && mem == SK_HOST) {
     cudaMemcpyAsync(f_out, df, b3, cudaMemcpyDeviceToHost, st);

@@ -53,16 +53,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   }
 }
 
-// 1/sqrt(x): the hardware's approximation y0 (about 20 bits, one instruction)
-// and one step of Householder's cubic iteration, y0 (1 + e/2 + 3/8 e^2) with
-// e = 1 - x y0^2; the term left out is below 2^-60. Overflowed x gives 0.
-__device__ __forceinline__ double rsqrt_fp64(double x) {
-  double y0;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
-  const double e = __double2hiint(x) < 0x7ff00000 ? fma(-x, y0 * y0, 1.0) : 0.0;
-  return fma(y0, e * fma(0.375, e, 0.5), y0);
-}
-
 template <int LAYER>
 __device__ __forceinline__ void far64(const double4_32a& G, const double4_32a& Nn, double dx,
                                       double dy, double dz, double r2, double* u) {
