@@ -181,7 +181,7 @@ int enqueue_prep(const EvalShape& s, const EvalBufs& b, double rho_T, double rho
                      b.tbbox_part, b.tbbox, b.meta + META_SCRATCH, s.small_sort_points, tst);
   launches += sort_launches(s.M);
   if (fp32)
-    launch_pack_targets32(b, s.n_delta, rho_T, rho_c, tst);
+    launch_pack_targets32(b, s.n_delta, rho_c, tst);
   else
     launch_pack_targets64(b, s.n_delta, tst);
   if (s.N > 0) {
@@ -209,7 +209,7 @@ int enqueue_eval(const EvalShape& s, const EvalBufs& b, double rho_T, double rho
   int launches = enqueue_prep(s, b, rho_T, rho_c, st, pf);
   if (ev) cudaEventRecord(ev[1], st);
   if (fp32) {
-    launch_pair32(s.layer, b, rho_T, scale, st, ev ? ev[2] : nullptr);  // with the finish
+    launch_pair32(s.layer, b, rho_T, rho_c, scale, st, ev ? ev[2] : nullptr);  // with the finish
     launches += b.fuse_finish ? 1 : 3;
   } else {
     launch_pair64(s.layer, b, scale, st);

@@ -796,7 +796,7 @@ __global__ void k_fmm_pack_tgt(const double* __restrict__ Y, const double* __res
                                int64_t n_delta, const int* __restrict__ tlist,
                                const int* __restrict__ toff, const int* __restrict__ tcount,
                                const int* __restrict__ block_box, const int* __restrict__ box_first,
-                               int tb, int64_t n_slots, double rho_T, double rho_c,
+                               int tb, int64_t n_slots, double rho_c,
                                float4* __restrict__ tgtF, double4_32a* __restrict__ tgt64,
                                int* __restrict__ perm) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -807,10 +807,7 @@ __global__ void k_fmm_pack_tgt(const double* __restrict__ Y, const double* __res
   const int64_t j = tlist[toff[i] + (real ? q : 0)];
   const double x = Y[3 * j], y = Y[3 * j + 1], z = Y[3 * j + 2];
   const double d = delta[n_delta == 1 ? 0 : j];
-  const double rc = rho_c * d, rt = rho_T * d;
-  tgtF[2 * t] = make_float4((float)x, (float)y, (float)z, (float)(1.0 / d));
-  tgtF[2 * t + 1] = real ? make_float4((float)(rc * rc), (float)(rt * rt), 0.f, 0.f)
-                         : make_float4(-1.f, -1.f, 0.f, 0.f);
+  write_tgt_record(tgtF + 2 * t, x, y, z, d, rho_c, real);
   tgt64[t] = make_double4_32a(x, y, z, d);
   perm[t] = real ? (int)j : -1;
 }
@@ -829,30 +826,40 @@ __global__ void __launch_bounds__(TPB32, MINB)
       a, it.x, p32::TileList{desc + it.y, it.z, it.w, TB, (int64_t)it.x * TB}, sm, ps);
 }
 
-// One CTA of G threads per target group of G targets (a thread per target):
-// each target's item partials in item order plus its FP64 near sum (the
-// near-sum scratch in dynamic shared memory); u at the target's original
-// index.
+// FMM_FIN_PARTS CTAs per target group of G targets: each target's item partials
+// plus its FP64 near sum (the near-sum scratch in dynamic shared memory); u at
+// the target's original index.
+constexpr int FMM_FIN_PARTS = 2, FMM_FIN_THREADS = 128;
 template <int G>
-__global__ void __launch_bounds__(G)
+__global__ void __launch_bounds__(FMM_FIN_THREADS)
     k_fmm_finish32(p32::OverflowArgs oa, p32::FinishArgs fa, const int* __restrict__ item_first,
                    int tb) {
-  extern __shared__ unsigned fsm[];
-  int cnt = p32::near_group<p32::SLayer, G>(
-      oa, fa, blockIdx.x, fsm, threadIdx.x, [&](int64_t t, double n0, double n1, double n2) {
-        const int64_t j = fa.perm[t];
-        if (j < 0) return;
-        const int64_t b = t / tb, l = t - b * tb;
+  extern __shared__ __align__(16) unsigned fsm[];
+  constexpr int KP = G / FMM_FIN_PARTS;
+  const int k0 = (int)(blockIdx.x % FMM_FIN_PARTS) * KP;
+  int cnt = p32::near_group<p32::SLayer, G, FMM_FIN_THREADS>(
+      oa, fa, blockIdx.x / FMM_FIN_PARTS, k0, k0 + KP, fsm,
+      reinterpret_cast<double*>(fsm + p32::near_warp_words(G)), threadIdx.x,
+      [&](int64_t t, bool valid, int sub, double n0, double n1, double n2) {
+        const int64_t j = valid ? fa.perm[t] : -1;
         double u0 = 0.0, u1 = 0.0, u2 = 0.0;
-        for (int it = item_first[b]; it < item_first[b + 1]; ++it) {
-          const double* p = fa.part + ((size_t)it * tb + l) * 3;
-          u0 += p[0];
-          u1 += p[1];
-          u2 += p[2];
+        if (j >= 0) {
+          const int64_t b = t / tb, l = t - b * tb;
+          for (int it = item_first[b] + sub; it < item_first[b + 1]; it += p32::FIN_SUBS) {
+            const double* p = fa.part + ((size_t)it * tb + l) * 3;
+            u0 += p[0];
+            u1 += p[1];
+            u2 += p[2];
+          }
         }
-        fa.u[3 * j] = u0 + n0;
-        fa.u[3 * j + 1] = u1 + n1;
-        fa.u[3 * j + 2] = u2 + n2;
+        u0 = p32::fin_sum(u0);
+        u1 = p32::fin_sum(u1);
+        u2 = p32::fin_sum(u2);
+        if (j >= 0 && sub == 0) {
+          fa.u[3 * j] = u0 + n0;
+          fa.u[3 * j + 1] = u1 + n1;
+          fa.u[3 * j + 2] = u2 + n2;
+        }
       });
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
   if ((threadIdx.x & 31) == 0 && cnt)
@@ -1248,12 +1255,12 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
           box, op->unit, Np, eqp, cv.phi, count, k, scale, near_slots, cv.srcF, cv.segbox);
       k_fmm_pack_tgt<<<nblk(m_slots), FMM_TPB, 0, st>>>(Y, D, n_delta, cv.tlist, cv.toffs,
                                                         cv.tcount, d_bb, d_bf, tb, m_slots,
-                                                        ctx->rho_T, ctx->rho_c, cv.tgtF,
+                                                        ctx->rho_c, cv.tgtF,
                                                         cv.tgt64, cv.perm);
       // 6. the pair sums of every item, the overflow rescans and the finish
-      p32::PairArgs a{cv.srcF, cv.segbox, cv.src_orig, cv.meta, cv.tgtF, cv.tgt64, m_slots, 1,
-                      cv.part, cv.near_cnt, cv.near_idx, cv.flags, (float)ctx->rho_T, 8.0f,
-                      nullptr};
+      p32::PairArgs a{cv.srcF, cv.segbox, cv.src_orig, cv.meta, cv.tgtF, m_slots, 1,
+                      cv.part, cv.near_cnt, cv.near_idx, cv.flags,
+                      near_ratio(ctx->rho_T, ctx->rho_c)};
       if (np32 == 2)
         launch_pair32_fmm<2>(a, d_it, d_de, n_items, st);
       else
@@ -1262,15 +1269,18 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
                            cv.near_cnt, X,        W,           F,       nullptr, scale,
                            cv.flags,  cv.near_ovf};
       oa.group = 64 * np32;
+      oa.rt_ratio = a.rt_ratio;
       k_fmm_overflow32<<<(unsigned)((m_slots * 32 + 255) / 256), 256, 0, st>>>(oa, m_slots);
       p32::FinishArgs fa{cv.tgt64, cv.perm, m_slots, 1, cv.part, cv.near_cnt, cv.near_idx,
                          cv.near_ovf, X, W, F, nullptr, scale, U, cv.flags};
       fa.group = 64 * np32;
-      const size_t fsmem = (size_t)p32::near_warp_words(fa.group) * 4;
+      const size_t fsmem = (size_t)p32::near_warp_words(fa.group) * 4 +
+                           FMM_FIN_THREADS * 3 * sizeof(double);
+      const unsigned fgrid = (unsigned)(m_slots / fa.group) * FMM_FIN_PARTS;
       if (np32 == 2)
-        k_fmm_finish32<128><<<(unsigned)(m_slots / 128), 128, fsmem, st>>>(oa, fa, d_if, tb);
+        k_fmm_finish32<128><<<fgrid, FMM_FIN_THREADS, fsmem, st>>>(oa, fa, d_if, tb);
       else
-        k_fmm_finish32<64><<<(unsigned)(m_slots / 64), 64, fsmem, st>>>(oa, fa, d_if, tb);
+        k_fmm_finish32<64><<<fgrid, FMM_FIN_THREADS, fsmem, st>>>(oa, fa, d_if, tb);
       ctx->stats = sk_eval_stats{};
       ctx->stats.n_tgt = n_tgt;
       ctx->stats.n_chunks = n_items;

@@ -110,6 +110,30 @@ __device__ __forceinline__ void write_sl_record(float4* o, float x, float y, flo
   o[1] = make_float4(-z, -z, g0, g0);
   o[2] = make_float4(g1, g1, g2, g2);
 }
+#endif
+
+#ifdef __CUDACC__
+// FP32 target record, two float4: (x, y, z, 1/delta) and (rho_c^2 delta^2,
+// then the residuals x - fl32(x), .. of the coordinates). The (hi, lo) split
+// is made once per target here: the FP64 conversions would otherwise be
+// repeated by every source chunk of the pair kernel, on an FP64 pipe that is
+// 64 times slower than the FP32 one. Padding targets (!real) get a radius of
+// -1. rho_T^2 delta^2 is taken from rho_c^2 delta^2 (near_radius2).
+__device__ __forceinline__ void write_tgt_record(float4* o, double x, double y, double z, double d,
+                                                 double rho_c, bool real) {
+  const float hx = (float)x, hy = (float)y, hz = (float)z;
+  const double rc = rho_c * d;
+  o[0] = make_float4(hx, hy, hz, (float)(1.0 / d));
+  o[1] = make_float4(real ? (float)(rc * rc) : -1.f, (float)(x - (double)hx),
+                     (float)(y - (double)hy), (float)(z - (double)hz));
+}
+
+// rho_T^2 delta^2 from the record's rho_c^2 delta^2; ratio = (rho_T / rho_c)^2.
+// The pair kernel and the overflow rescan both call this.
+__device__ __forceinline__ float near_radius2(float rc2, float ratio) {
+  return __fmul_rn(rc2, ratio);
+}
+
 // 1/sqrt(x): the hardware's approximation y0 (about 20 bits, one instruction)
 // and one step of Householder's cubic iteration, y0 (1 + e/2 + 3/8 e^2) with
 // e = 1 - x y0^2; the term left out is below 2^-60. Overflowed x gives 0.
@@ -119,7 +143,37 @@ __device__ __forceinline__ double rsqrt_fp64(double x) {
   const double e = __double2hiint(x) < 0x7ff00000 ? fma(-x, y0 * y0, 1.0) : 0.0;
   return fma(y0, e * fma(0.375, e, 0.5), y0);
 }
+
+// 1/x the same way (reciprocal approximation and one cubic step).
+__device__ __forceinline__ double rcp_fp64(double x) {
+  double y0;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+  const double e = fma(-x, y0, 1.0);
+  return fma(y0, fma(e, e, e), y0);
+}
+
+// (float)x, truncated, by integer instructions; 0 for |x| below 2^-126. x must
+// be finite and below 2^128.
+__device__ __forceinline__ float narrow(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const unsigned mag = hi & 0x7fffffffu;
+  if (mag < 0x38100000u) return 0.f;
+  return __uint_as_float((hi & 0x80000000u) | ((mag - 0x38000000u) << 3) | (lo >> 29));
+}
+
+// (double)w by integer instructions (a conversion would take the FP64 pipe).
+__device__ __forceinline__ double widen(float w) {
+  const unsigned b = __float_as_uint(w);
+  if (((b >> 23) & 0xffu) - 1u >= 254u) return (double)w;  // zero, subnormal, inf, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)),
+                          (int)(b << 29));
+}
 #endif
+
+// (rho_T / rho_c)^2 for near_radius2
+inline float near_ratio(double rho_T, double rho_c) {
+  return (float)((rho_T / rho_c) * (rho_T / rho_c));
+}
 
 // Padding sources sit this far away, with zero density.
 constexpr float PAD_POS = 1.0e15f;
@@ -175,7 +229,7 @@ struct EvalBufs {
   const char* factors64 = nullptr;    // FP64 factor tables (the context's)
   float4* segbox = nullptr;       // per segment: lo, hi
   int* tgt_perm = nullptr;        // sorted target -> original index
-  float4* tgtF = nullptr;         // FP32 sorted targets: (x, y, z, 1/delta), (rc2, rt2, 0, 0)
+  float4* tgtF = nullptr;         // FP32 sorted targets (write_tgt_record)
   double4_32a* tgt64 = nullptr;       // FP64 sorted targets: (x, y, z, delta)
   // accumulation
   double* part = nullptr;         // [n_chunks][M_pad][3]
@@ -316,8 +370,7 @@ int launch_sort_pairs(uint32_t* keys_a, uint32_t* keys_b, int* vals_a, int* vals
                       int bits, uint32_t* hist, cudaStream_t st);
 void launch_pack_sources32(int layer, const EvalBufs& b, double scale, cudaStream_t st);
 void launch_pack_sources64(int layer, const EvalBufs& b, double scale, cudaStream_t st);
-void launch_pack_targets32(const EvalBufs& b, int64_t n_delta, double rho_T, double rho_c,
-                           cudaStream_t st);
+void launch_pack_targets32(const EvalBufs& b, int64_t n_delta, double rho_c, cudaStream_t st);
 void launch_pack_targets64(const EvalBufs& b, int64_t n_delta, cudaStream_t st);
 int sort_grid_blocks(int64_t n);
 
@@ -326,8 +379,8 @@ int sort_grid_blocks(int64_t n);
 // FP64 near sums, chunk merge, output write): fused into the pair kernel when
 // b.fuse_finish, else two more launches. pair_end (optional) is recorded
 // after the pair kernel, before any finish launch.
-void launch_pair32(int layer, const EvalBufs& b, double rho_T, double scale, cudaStream_t st,
-                   cudaEvent_t pair_end = nullptr);
+void launch_pair32(int layer, const EvalBufs& b, double rho_T, double rho_c, double scale,
+                   cudaStream_t st, cudaEvent_t pair_end = nullptr);
 void launch_pair64(int layer, const EvalBufs& b, double scale, cudaStream_t st);
 void launch_finish64(const EvalBufs& b, cudaStream_t st);
 

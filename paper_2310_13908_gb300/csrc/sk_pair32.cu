@@ -13,13 +13,13 @@ using namespace p32;
 // beside other CTAs' FP32 pair work instead of in kernels of its own. With
 // few blocks a block's finish on one CTA would become the tail, so the plain
 // kernel is followed by the finish kernels below.
-template <class L, int NP, int MINB>
-__global__ void __launch_bounds__(TPB32, MINB) k_pair32(PairArgs a) {
+template <class L, int NP, int TPB, int MINB>
+__global__ void __launch_bounds__(TPB, MINB) k_pair32(PairArgs a) {
   extern __shared__ __align__(128) float4 sm[];
-  __shared__ PipeSmem<pair_stages<L, NP>()> ps;
+  __shared__ PipeSmem<pair_stages<L, NP, TPB>()> ps;
   if (threadIdx.x == 0) ps.initialized = 0;
   const int tb = blockIdx.x / a.n_chunks, ch = blockIdx.x % a.n_chunks;
-  pair_item<L, NP>(a, tb, chunk_tiles(a, ch), sm, ps);
+  pair_item<L, NP, TPB>(a, tb, chunk_tiles(a, ch), sm, ps);
 }
 
 template <class L, int NP, int MINB>
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(TPB32, MINB)
   // the source stages are free now: the finish buckets the near lists there
   static_assert(pair_smem_bytes<L, NP>() / 4 >= (size_t)(TPB32 / 32) * near_warp_words(64 * NP),
                 "finish scratch");
-  finish_block<L>(oa, fa, M, (int64_t)tb * TB, TB, reinterpret_cast<unsigned*>(sm));
+  finish_block<L, 64 * NP>(oa, fa, M, (int64_t)tb * TB, TB, reinterpret_cast<unsigned*>(sm));
 }
 
 template <class L>
@@ -55,69 +55,88 @@ __global__ void k_overflow32(OverflowArgs a, int64_t M) {
   overflow_target<L>(a, t);
 }
 
-// Separate finish for grids too small to fuse it: one CTA of G threads per
-// target group of G targets (a thread per target), the near-sum scratch in
-// dynamic shared memory.
+// Separate finish for grids too small to fuse it: FIN_PARTS CTAs per target
+// group of G targets, each with its share of the targets (and the whole list,
+// of which it keeps its own), the near-sum scratch in dynamic shared memory.
+// Bound by the FP64 pipe (60% busy) and the latency of its phases; small grids
+// by how many SMs get a share. Against one CTA per group with a thread per
+// target (single layer): 104 -> 72 us at 24,576 targets (64 chunks, 12 near pairs
+// per target), 47 -> 16 us at 1,944, 61 -> 22 us at 5,766; one warp per share
+// instead of four took 112 us at 24,576 targets.
+constexpr int FIN_PARTS = 4, FIN_THREADS = 128;
 template <class L, int G>
-__global__ void __launch_bounds__(G) k_finish32(OverflowArgs oa, FinishArgs a, int64_t M) {
-  extern __shared__ unsigned fsm[];
-  const int64_t t0 = (int64_t)blockIdx.x * G;
-  int cnt = near_group<L, G>(oa, a, blockIdx.x, fsm, threadIdx.x,
-                             [&](int64_t t, double n0, double n1, double n2) {
-                               if (t < M) finish_merge(a, t, n0, n1, n2);
-                             });
+__global__ void __launch_bounds__(FIN_THREADS) k_finish32(OverflowArgs oa, FinishArgs a,
+                                                           int64_t M) {
+  extern __shared__ __align__(16) unsigned fsm[];
+  constexpr int KP = G / FIN_PARTS;
+  const int64_t g = blockIdx.x / FIN_PARTS;
+  const int k0 = (int)(blockIdx.x % FIN_PARTS) * KP;
+  int cnt = near_group<L, G, FIN_THREADS>(
+      oa, a, g, k0, k0 + KP, fsm, reinterpret_cast<double*>(fsm + near_warp_words(G)), threadIdx.x,
+      [&](int64_t t, bool valid, int sub, double n0, double n1, double n2) {
+        finish_merge(a, t, valid && t < M, sub, n0, n1, n2);
+      });
   // count near pairs: one atomic per warp
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
   if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(a.flags + FLAG_NEAR_PAIRS, (unsigned long long)cnt);
-  __syncthreads();  // this group's targets are finished: their scratch is dead
-  discard_block_scratch(a, t0, G, threadIdx.x, blockDim.x);
+  __syncthreads();  // these targets are finished: their partials are dead
+  discard_block_partials(a, g * G + k0, KP, threadIdx.x, blockDim.x);
 }
 
 }  // namespace
 
 template <class L, int NP>
-void launch_pair32_t(const EvalBufs& b, float rho_lo, float rho_hi, double scale, cudaStream_t st,
-                     cudaEvent_t pair_end) {
+void launch_pair32_t(const EvalBufs& b, float rt_ratio, double scale,
+                     cudaStream_t st, cudaEvent_t pair_end) {
   constexpr int MINB = NP == 2 ? PAIR32_MINB_NP2 : PAIR32_MINB_NP1;
   const unsigned grid = (unsigned)((b.M_pad / (TPB32 * 2 * NP)) * b.n_chunks);
   const size_t smem = pair_smem_bytes<L, NP>();
-  PairArgs a{b.srcF,  b.segbox,   b.src_orig, b.meta,     b.tgtF,  b.tgt64, b.M_pad,
-             b.n_chunks, b.part, b.near_cnt, b.near_idx, b.flags, rho_lo, rho_hi, b.srcLo};
+  PairArgs a{b.srcF,  b.segbox,   b.src_orig, b.meta,     b.tgtF, b.M_pad,
+             b.n_chunks, b.part, b.near_cnt, b.near_idx, b.flags, rt_ratio, b.srcLo};
   OverflowArgs oa{b.srcF, b.segbox, b.src_orig, b.meta,  b.tgtF,  b.tgt64,     b.near_cnt,
                   b.src_xyz, b.src_w, b.dens,   b.nrm, scale, b.flags, b.near_ovf};
   FinishArgs fa{b.tgt64, b.tgt_perm, b.M_pad, b.n_chunks, b.part, b.near_cnt, b.near_idx,
                 b.near_ovf, b.src_xyz, b.src_w, b.dens, b.nrm, scale, b.u, b.flags};
   oa.group = fa.group = 64 * NP;
+  oa.rt_ratio = rt_ratio;
   if (b.fuse_finish) {
     cudaFuncSetAttribute(k_pair32_fused<L, NP, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
     k_pair32_fused<L, NP, MINB><<<grid, TPB32, smem, st>>>(a, oa, fa, b.tb_done, b.M);
     if (pair_end) cudaEventRecord(pair_end, st);
   } else {
-    cudaFuncSetAttribute(k_pair32<L, NP, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-    k_pair32<L, NP, MINB><<<grid, TPB32, smem, st>>>(a);
+    // One pair per lane, single layer: CTAs of 128 threads. A CTA's warps meet
+    // few or many segments inside rho_c delta, and the SM waits for the
+    // slowest; smaller CTAs wait less (pair kernel at 128 / 256 threads: 1,944
+    // nodes 60 / 68 us, 24,576 nodes 373 / 385 us, 96,774 sources x 5,766
+    // targets 418 / 430 us; 64 threads: slower from 24,576 nodes on). The
+    // stresslet's larger records leave room for too few of them: 417 / 405 us.
+    constexpr int TPB = NP == 1 && L::V == V_SL ? 128 : TPB32;
+    constexpr size_t smem1 = pair_smem_bytes<L, NP, TPB>();
+    const auto k = k_pair32<L, NP, TPB, MINB * (TPB32 / TPB)>;
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
+    k<<<grid * (TPB32 / TPB), TPB, smem1, st>>>(a);
     if (pair_end) cudaEventRecord(pair_end, st);
     k_overflow32<L><<<(unsigned)((b.M * 32 + 255) / 256), 256, 0, st>>>(oa, b.M);
     constexpr int G = 64 * NP;
-    const size_t fsmem = (size_t)near_warp_words(G) * sizeof(unsigned);
-    k_finish32<L, G><<<(unsigned)(b.M_pad / G), G, fsmem, st>>>(oa, fa, b.M);
+    const size_t fsmem = (size_t)near_warp_words(G) * sizeof(unsigned) + FIN_THREADS * 3 * sizeof(double);
+    k_finish32<L, G><<<(unsigned)(b.M_pad / G * FIN_PARTS), FIN_THREADS, fsmem, st>>>(oa, fa, b.M);
   }
 }
 
-void launch_pair32(int layer, const EvalBufs& b, double rho_T, double scale, cudaStream_t st,
-                   cudaEvent_t pair_end) {
-  const float rho_lo = (float)rho_T, rho_hi = 8.0f;
+void launch_pair32(int layer, const EvalBufs& b, double rho_T, double rho_c, double scale,
+                   cudaStream_t st, cudaEvent_t pair_end) {
+  const float ratio = near_ratio(rho_T, rho_c);
   if (layer == LAYER_SL) {
     if (b.pair_np == 2)
-      launch_pair32_t<SLayer, 2>(b, rho_lo, rho_hi, scale, st, pair_end);
+      launch_pair32_t<SLayer, 2>(b, ratio, scale, st, pair_end);
     else
-      launch_pair32_t<SLayer, 1>(b, rho_lo, rho_hi, scale, st, pair_end);
+      launch_pair32_t<SLayer, 1>(b, ratio, scale, st, pair_end);
   } else {
     if (b.pair_np == 2)
-      launch_pair32_t<DLayer, 2>(b, rho_lo, rho_hi, scale, st, pair_end);
+      launch_pair32_t<DLayer, 2>(b, ratio, scale, st, pair_end);
     else
-      launch_pair32_t<DLayer, 1>(b, rho_lo, rho_hi, scale, st, pair_end);
+      launch_pair32_t<DLayer, 1>(b, ratio, scale, st, pair_end);
   }
 }
 

@@ -72,11 +72,6 @@ __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); 
 // read-only path. ld.global.cg goes to L2, which every write reaches. A
 // kernel launched per evaluation starts with clean L1 and keeps its ordinary
 // loads.
-__device__ __forceinline__ double4_32a ldcg4d(const double4_32a* p) {
-  const double2* q = reinterpret_cast<const double2*>(p);
-  const double2 a = __ldcg(q), b = __ldcg(q + 1);
-  return make_double4_32a(a.x, a.y, b.x, b.y);
-}
 
 // ---- bulk async copy + mbarrier helpers (bounded waits) --------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -117,10 +112,20 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
 }
 
 // ---- per-lane target state --------------------------------------------------
+// in shared memory: TGT_SLOTS float4 per f32x2 pair and thread (see pair_smem_bytes)
+constexpr int TGT_SLOTS = 5;
 // x, y, z: the pair's targets relative to the current segment's frame,
 // recomputed per segment from the targets' FP32 (hi, lo) splits.
 struct Tgt2 {
   float2 x, y, z, idl, rc2, rt2;
+  // 1/delta and the squared radii, from the pair's column (ts of pair_smem_bytes)
+  template <int TPB>
+  __device__ __forceinline__ void load_radii(const float4* ts) {
+    const float4 q = ts[3 * TPB], r = ts[4 * TPB];
+    idl = make_float2(q.x, q.y);
+    rc2 = make_float2(q.z, q.w);
+    rt2 = make_float2(r.x, r.y);
+  }
 };
 
 // A target coordinate x = hi + lo (hi = fl32(x), lo = fl32(x - hi)) relative
@@ -163,52 +168,74 @@ __device__ __forceinline__ float box_margin(float coord_max, float rc) {
 // of one warp of the pair kernel (group g = first target / (64 * NP)). An
 // entry is (k << NEAR_SRC_BITS) | jo, k the target's place in the group and
 // jo the source's original index. The warp appends the near pairs of one
-// source together: one atomic per warp and source, and consecutive slots, so
-// the group's list fills whole 32-byte sectors. (Entries appended one by one
-// to per-target lists leave a partly written sector per target, which L2
-// completes from DRAM when the finish reads it.) near_bits holds bit 2p + h
-// for the lane's target 64p + 32h + lane. A list longer than NEAR_K * 64 * NP
+// segment of 32 sources together: one atomic per warp and segment, and
+// consecutive slots, so the group's list fills whole 32-byte sectors. (Entries
+// appended one by one to per-target lists leave a partly written sector per
+// target, which L2 completes from DRAM when the finish reads it; one append
+// per source put the atomic's latency, about a thousand cycles, into every
+// source iteration with a near pair.) A list longer than NEAR_K * 64 * NP
 // entries keeps counting but stores no more; the group's targets then take
 // the rescan of overflow_target.
+//
+// A lane's near pairs with one segment: bit j of m[2p + h] is set for source
+// j and the lane's target 64p + 32h + lane.
+template <int NP>
+struct NearMask {
+  unsigned m[2 * NP];
+};
+
 template <int NP, bool kFresh>
-__device__ __noinline__ void near_append_list(unsigned near_bits, int lane, int64_t g,
-                                              const int* jo_at, int* __restrict__ cnt,
-                                              unsigned* __restrict__ idx,
+__device__ __noinline__ void near_append_list(NearMask<NP> nm, int64_t g, const int* orig,
+                                              int* __restrict__ cnt, unsigned* __restrict__ idx,
                                               unsigned long long* __restrict__ flags) {
   constexpr int CAP = NEAR_K * 64 * NP;
-  const unsigned jo = (unsigned)(kFresh ? __ldcg(jo_at) : *jo_at);
-  const unsigned lt = (1u << lane) - 1u;
-  int total = 0;
+  const int lane = threadIdx.x & 31;
+  int n = 0;
 #pragma unroll
-  for (int b = 0; b < 2 * NP; ++b) total += __popc(__ballot_sync(FULL, (near_bits >> b) & 1u));
+  for (int b = 0; b < 2 * NP; ++b) n += __popc(nm.m[b]);
+  int end = n;  // inclusive scan over the lanes
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(FULL, end, o);
+    if (lane >= o) end += y;
+  }
+  const int total = __shfl_sync(FULL, end, 31);
   int base = 0;
   if (lane == 0) {
     base = atomicAdd(cnt + g, total);
     // the group's targets will be rescanned: count them
     if (base <= CAP && base + total > CAP) atomicAdd(flags + FLAG_OVERFLOW, 64ull * NP);
   }
-  base = __shfl_sync(FULL, base, 0);
+  int slot = __shfl_sync(FULL, base, 0) + end - n;
   unsigned* __restrict__ list = idx + (size_t)g * CAP;
-  // slots in (bit, lane) order: the ballots again, so that no offsets stay live
+  const int own = kFresh ? __ldcg(orig + lane) : orig[lane];  // source `lane` of the segment
 #pragma unroll
-  for (int b = 0; b < 2 * NP; ++b) {
-    const unsigned m = __ballot_sync(FULL, (near_bits >> b) & 1u);
-    const int slot = base + __popc(m & lt);
-    if (((near_bits >> b) & 1u) && slot < CAP)
-      list[slot] = ((unsigned)(64 * (b >> 1) + 32 * (b & 1) + lane) << NEAR_SRC_BITS) | jo;
-    base += __popc(m);
+  for (int p = 0; p < NP; ++p) {
+    unsigned long long m = ((unsigned long long)nm.m[2 * p + 1] << 32) | nm.m[2 * p];
+    while (__any_sync(FULL, m != 0ull)) {
+      const int bit = m ? __ffsll((long long)m) - 1 : 0;  // 32 h + source
+      const unsigned jo = (unsigned)__shfl_sync(FULL, own, bit & 31);
+      if (m) {
+        if (slot < CAP)
+          list[slot] = ((unsigned)(64 * p + (bit & 32) + lane) << NEAR_SRC_BITS) | jo;
+        ++slot;
+        m &= m - 1ull;
+      }
+    }
   }
 }
 
-// Out of line beyond the vote: few general-path sources have a near pair,
+// Out of line beyond the vote: few general-path segments have a near pair,
 // and the append's registers then do not weigh on the pair loop.
 template <int NP, bool kFresh>
-__device__ __forceinline__ void near_append_warp(unsigned near_bits, int lane, int64_t g,
-                                                 const int* jo_at, int* __restrict__ cnt,
+__device__ __forceinline__ void near_append_warp(const NearMask<NP>& nm, int64_t g,
+                                                 const int* orig, int* __restrict__ cnt,
                                                  unsigned* __restrict__ idx,
                                                  unsigned long long* __restrict__ flags) {
-  if (__any_sync(FULL, near_bits))
-    near_append_list<NP, kFresh>(near_bits, lane, g, jo_at, cnt, idx, flags);
+  unsigned any = 0;
+#pragma unroll
+  for (int b = 0; b < 2 * NP; ++b) any |= nm.m[b];
+  if (__any_sync(FULL, any)) near_append_list<NP, kFresh>(nm, g, orig, cnt, idx, flags);
 }
 
 // ---- layer policies ---------------------------------------------------------
@@ -250,7 +277,7 @@ struct SLayer {
   // FP32 closed forms at rho (Sec. 3.4), with erf(rho) = 1 - exp(-rho^2) E(rho):
   // s = 1 - exp(-rho^2) (E(rho) + (2 / (3 sqrt(pi))) rho q(rho)), q the
   // factor's polynomial; one exponential and the fitted E (sk_erfc_scaled.h)
-  // instead of erff and an exponential. The caller clamps rho into range.
+  // instead of erff and an exponential. rho in [0, 8].
   __device__ __forceinline__ static void smooth(float rho, float& s1, float& s2) {
     const float p2 = rho * rho;
     const float e = __expf(-p2);
@@ -323,60 +350,36 @@ __device__ __forceinline__ void pair_d(const Tgt2& T, float2 nx, float2 ny, floa
 // decided on the FP32 difference r2 (the test of the far loop and of the
 // overflow rescan). rho and the kernel use (dx, dy, dz) and r2k, which equal
 // the FP32 difference and r2 except where pair_general corrected them.
+// A near pair (rho < rho_T) sets `bit` in m0 (component x) or m1 (component y).
+constexpr float RHO_HI = 8.0f;
 template <class L>
-__device__ __forceinline__ unsigned pair_general_regimes(const typename L::Src& S, const Tgt2& T,
-                                                         float2 dx, float2 dy, float2 dz,
-                                                         float2 r2, float2 r2k, float2* U,
-                                                         float rho_lo, float rho_hi) {
-  float2 ri = make_float2(rsq(r2k.x), rsq(r2k.y));
-  float2 sa = make_float2(1.f, 1.f), sb = make_float2(1.f, 1.f);
-  unsigned near_bits = 0;
-  // component x
-  {
-    const bool vn = r2.x < T.rt2.x;
-    const bool in = !vn && r2.x < T.rc2.x;
-    if (vn) {
-      near_bits |= 1u;
-      ri.x = 0.f;
-    }
-    float rho = fminf(fmaxf(r2k.x * ri.x * T.idl.x, rho_lo), rho_hi);
-    float a, b;
-    L::smooth(rho, a, b);
-    if (in) {
-      sa.x = a;
-      sb.x = b;
-    }
-  }
-  {
-    const bool vn = r2.y < T.rt2.y;
-    const bool in = !vn && r2.y < T.rc2.y;
-    if (vn) {
-      near_bits |= 2u;
-      ri.y = 0.f;
-    }
-    float rho = fminf(fmaxf(r2k.y * ri.y * T.idl.y, rho_lo), rho_hi);
-    float a, b;
-    L::smooth(rho, a, b);
-    if (in) {
-      sa.y = a;
-      sb.y = b;
-    }
-  }
+__device__ __forceinline__ void pair_general_regimes(const typename L::Src& S, const Tgt2& T,
+                                                     float2 dx, float2 dy, float2 dz, float2 r2,
+                                                     float2 r2k, float2* U, unsigned bit,
+                                                     unsigned& m0, unsigned& m1) {
+  // rho beyond rho_c becomes rho_hi = 8, where exp(-rho^2) < 2^-90 makes every
+  // factor exactly 1; a near pair gets ri = 0, hence rho = 0 and no sum
+  const bool n0 = r2.x < T.rt2.x, n1 = r2.y < T.rt2.y;
+  const float2 ri = make_float2(n0 ? 0.f : rsq(r2k.x), n1 ? 0.f : rsq(r2k.y));
+  const float2 rho = mul2(mul2(r2k, ri), T.idl);
+  float2 sa, sb;
+  L::smooth(r2.x < T.rc2.x ? rho.x : RHO_HI, sa.x, sb.x);
+  L::smooth(r2.y < T.rc2.y ? rho.y : RHO_HI, sa.y, sb.y);
   L::general(S, dx, dy, dz, ri, sa, sb, U);
-  return near_bits;
+  if (n0) m0 |= bit;
+  if (n1) m1 |= bit;
 }
 
 // For L::kExactNear, (cx, cy, cz) is the residual that makes the FP32
 // difference exact: pairs with rho_T <= rho < rho_c take the corrected
 // difference; the others keep the FP32 one, so a pair at or beyond rho_c
 // still reproduces the far formula bit for bit.
-// Returns the pair's near bits (x component: 1, y component: 2).
 template <class L>
-__device__ __forceinline__ unsigned pair_general(const typename L::Src& S, const Tgt2& T,
-                                                 float2 dx, float2 dy, float2 dz, float2 r2,
-                                                 float2* U, float rho_lo, float rho_hi,
-                                                 float2 cx = float2{}, float2 cy = float2{},
-                                                 float2 cz = float2{}) {
+__device__ __forceinline__ void pair_general(const typename L::Src& S, const Tgt2& T, float2 dx,
+                                             float2 dy, float2 dz, float2 r2, float2* U,
+                                             unsigned bit, unsigned& m0, unsigned& m1,
+                                             float2 cx = float2{}, float2 cy = float2{},
+                                             float2 cz = float2{}) {
   if constexpr (L::kExactNear) {
     const bool in0 = r2.x >= T.rt2.x && r2.x < T.rc2.x;
     const bool in1 = r2.y >= T.rt2.y && r2.y < T.rc2.y;
@@ -386,9 +389,9 @@ __device__ __forceinline__ unsigned pair_general(const typename L::Src& S, const
     dy = make_float2(in0 ? ey.x : dy.x, in1 ? ey.y : dy.y);
     dz = make_float2(in0 ? ez.x : dz.x, in1 ? ez.y : dz.y);
     const float2 r2k = make_float2(in0 ? er2.x : r2.x, in1 ? er2.y : r2.y);
-    return pair_general_regimes<L>(S, T, dx, dy, dz, r2, r2k, U, rho_lo, rho_hi);
+    pair_general_regimes<L>(S, T, dx, dy, dz, r2, r2k, U, bit, m0, m1);
   } else {
-    return pair_general_regimes<L>(S, T, dx, dy, dz, r2, r2, U, rho_lo, rho_hi);
+    pair_general_regimes<L>(S, T, dx, dy, dz, r2, r2, U, bit, m0, m1);
   }
 }
 
@@ -404,8 +407,6 @@ __device__ __forceinline__ void two_sum_merge(float2* U, float2* HI, float2* LO)
   }
 }
 
-// per-thread target state: TGT_SLOTS float4 per f32x2 pair (see pair_smem_bytes)
-constexpr int TGT_SLOTS = 5;
 // A segment is wide for a target when its frame's half extent exceeds this
 // many of the target's delta (see pair_item's general branch).
 constexpr float WIDE_FRAME = 4.0f;
@@ -421,50 +422,128 @@ struct LaneTgt {
   Tgt2 t[NP];
 };
 
+// The box of a warp's targets and the squared distance (with margins) within
+// which a source may have a pair inside rho_c delta with one of them: seven
+// numbers, kept one per lane in the warp's target columns (component z of slot
+// 4 of the first target pair), so that they take no registers in the far loop.
+struct WarpBox {
+  float lo[3], hi[3], r2;
+  // ts: the calling thread's column
+  template <int TPB>
+  __device__ __forceinline__ static WarpBox load(const float4* ts) {
+    const float* b = reinterpret_cast<const float*>(ts - (threadIdx.x & 31) + 4 * TPB) + 2;
+    return {{b[0], b[4], b[8]}, {b[12], b[16], b[20]}, b[24]};
+  }
+  // squared distance from the box to [l, h] (per axis), at most r2?
+  __device__ __forceinline__ bool reaches(float3 l, float3 h) const {
+    const float dx = fmaxf(0.f, fmaxf(l.x - hi[0], lo[0] - h.x));
+    const float dy = fmaxf(0.f, fmaxf(l.y - hi[1], lo[1] - h.y));
+    const float dz = fmaxf(0.f, fmaxf(l.z - hi[2], lo[2] - h.z));
+    return dx * dx + dy * dy + dz * dz < r2;
+  }
+};
+
+// Sources of a segment that may have such a pair: lane j tests source j
+// against the box, one step for the 32 sources. (sx, sy, sz): the segment's
+// frame, to which the record's position is relative.
+template <int V>
+__device__ __forceinline__ unsigned sources_near_box(const WarpBox& wb, const float4* SS, float sx,
+                                                     float sy, float sz) {
+  const float4* r = SS + (threadIdx.x & 31) * V;
+  const float4 a = r[0];  // {-x, -x, -y, -y}
+  const float3 x = make_float3(sx - a.x, sy - a.z, sz - r[1].x);
+  return __ballot_sync(FULL, wb.reaches(x, x));
+}
+
+// Four consecutive sources of a segment by the far formula.
+template <class L, int NP>
+__device__ __forceinline__ void far_four(LaneAcc<NP>& acc, const LaneTgt<NP>& tg,
+                                         const float4* SS) {
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const typename L::Src src = L::load(SS + j * L::V);
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      float2 dx, dy, dz, r2;
+      pair_d(tg.t[p], src.nx, src.ny, src.nz, dx, dy, dz, r2);
+      L::far(src, dx, dy, dz, r2, acc.u[p]);
+    }
+  }
+}
+
 // The general loop over the 32 sources of one segment near the warp's
-// targets: per source and target pair p, the far formula unless some lane's
-// pair p lies inside rho_c delta, then the regimes (which give the far
-// formula's bits for pairs beyond rho_c, so the choice per pair changes no
-// result) and the warp's near-pair append. Out of line:
-// its registers do not weigh on the far loop, and such segments are few (the
-// ones within rho_c delta of the warp's box).
-template <class L, int NP, bool kFresh>
+// targets, in source order. Sources that the box test clears run the far
+// formula, four at a time where it clears four in a row, without a vote; for
+// the others, per target pair p, the far formula unless some
+// lane's pair p lies inside rho_c delta, then the regimes (which give the far
+// formula's bits for pairs beyond rho_c, so neither choice changes a result).
+// The warp appends the segment's near pairs at the end. Out of line: its
+// registers do not weigh on the far loop. On a cell of 24,576 nodes 27% of the
+// (warp, segment) visits come here and about half of their sources are
+// cleared; they are half of the pair kernel's time (a voted source costs about
+// four far ones). Against a vote and an append per source: pair kernel 465 ->
+// 373 us there, 139 -> 60 us at 1,944 nodes, 580 -> 418 us for 96,774 sources x
+// 5,766 targets.
+template <class L, int NP, int TPB, bool kFresh>
 __device__ __noinline__ LaneAcc<NP> general_segment(LaneAcc<NP> acc, LaneTgt<NP> tg,
+                                                    const float4* ts, float sx, float sy, float sz,
                                                     const float4* SS, const int* orig,
                                                     int64_t group, int* near_cnt,
                                                     unsigned* near_idx,
-                                                    unsigned long long* flags, float rho_lo,
-                                                    float rho_hi) {
+                                                    unsigned long long* flags) {
   constexpr int V = L::V;
-  const int lane = threadIdx.x & 31;
+  const unsigned near_src = sources_near_box<V>(WarpBox::load<TPB>(ts), SS, sx, sy, sz);
+#pragma unroll
+  for (int p = 0; p < NP; ++p) tg.t[p].template load_radii<TPB>(ts + p * TGT_SLOTS * TPB);
+  NearMask<NP> nm{};
 #pragma unroll 1
-  for (int j = 0; j < SEG; ++j) {
-    const typename L::Src src = L::load(SS + j * V);
-    float2 dx[NP], dy[NP], dz[NP], r2[NP];
-    unsigned inr = 0;
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      pair_d(tg.t[p], src.nx, src.ny, src.nz, dx[p], dy[p], dz[p], r2[p]);
-      inr |= (__any_sync(FULL, (r2[p].x < tg.t[p].rc2.x) | (r2[p].y < tg.t[p].rc2.y)) ? 1u : 0u)
-             << p;
+  for (int g = 0; g < SEG; g += 4) {
+    if (((near_src >> g) & 15u) == 0u) {
+      far_four<L, NP>(acc, tg, SS + g * V);
+      continue;
     }
-    if (inr) {
-      unsigned near_bits = 0;
+    if constexpr (NP == 1) {
+      // two sources at a time: two independent chains per warp
+#pragma unroll 1
+      for (int j = g; j < g + 4; j += 2) {
+        typename L::Src src[2];
+        float2 dx[2], dy[2], dz[2], r2[2];
+        bool in = false;
 #pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        if ((inr >> p) & 1u)
-          near_bits |= pair_general<L>(src, tg.t[p], dx[p], dy[p], dz[p], r2[p], acc.u[p],
-                                       rho_lo, rho_hi)
-                       << (2 * p);
-        else
-          L::far(src, dx[p], dy[p], dz[p], r2[p], acc.u[p]);
+        for (int i = 0; i < 2; ++i) {
+          src[i] = L::load(SS + (j + i) * V);
+          pair_d(tg.t[0], src[i].nx, src[i].ny, src[i].nz, dx[i], dy[i], dz[i], r2[i]);
+          in |= (r2[i].x < tg.t[0].rc2.x) | (r2[i].y < tg.t[0].rc2.y);
+        }
+        if (((near_src >> j) & 3u) && __any_sync(FULL, in)) {
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+            pair_general<L>(src[i], tg.t[0], dx[i], dy[i], dz[i], r2[i], acc.u[0], 1u << (j + i),
+                            nm.m[0], nm.m[1]);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 2; ++i) L::far(src[i], dx[i], dy[i], dz[i], r2[i], acc.u[0]);
+        }
       }
-      near_append_warp<NP, kFresh>(near_bits, lane, group, orig + j, near_cnt, near_idx, flags);
     } else {
+#pragma unroll 1
+      for (int j = g; j < g + 4; ++j) {
+        const typename L::Src src = L::load(SS + j * V);
+        const bool maybe = (near_src >> j) & 1u;
 #pragma unroll
-      for (int p = 0; p < NP; ++p) L::far(src, dx[p], dy[p], dz[p], r2[p], acc.u[p]);
+        for (int p = 0; p < NP; ++p) {
+          float2 dx, dy, dz, r2;
+          pair_d(tg.t[p], src.nx, src.ny, src.nz, dx, dy, dz, r2);
+          if (maybe && __any_sync(FULL, (r2.x < tg.t[p].rc2.x) | (r2.y < tg.t[p].rc2.y)))
+            pair_general<L>(src, tg.t[p], dx, dy, dz, r2, acc.u[p], 1u << j, nm.m[2 * p],
+                            nm.m[2 * p + 1]);
+          else
+            L::far(src, dx, dy, dz, r2, acc.u[p]);
+        }
+      }
     }
   }
+  near_append_warp<NP, kFresh>(nm, group, orig, near_cnt, near_idx, flags);
   return acc;
 }
 
@@ -476,13 +555,14 @@ __device__ __noinline__ LaneAcc<NP> general_segment(LaneAcc<NP> acc, LaneTgt<NP>
 // general loop computes, in the same order, so the accumulators come out bit
 // for bit as there. Out of line: its registers do not weigh on the pair loop,
 // and wide segments are rare on dense surfaces.
-template <class L, int NP, bool kFresh>
+template <class L, int NP, int TPB, bool kFresh>
 __device__ __noinline__ LaneAcc<NP> exact_segment(
-    LaneAcc<NP> acc, LaneTgt<NP> tg, const float4* SS, const float4* __restrict__ ylo,
-    const int* orig, const float4* ts, float sx, float sy, float sz, float hs, int64_t group,
-    int* near_cnt, unsigned* near_idx, unsigned long long* flags, float rho_lo, float rho_hi) {
+    LaneAcc<NP> acc, LaneTgt<NP> tg, const float4* SS,
+    const float4* __restrict__ ylo, const int* orig, const float4* ts, float sx, float sy, float sz, float hs, int64_t group,
+    int* near_cnt, unsigned* near_idx, unsigned long long* flags) {
   constexpr int V = L::V;
-  const int lane = threadIdx.x & 31;
+  const unsigned near_src = sources_near_box<V>(WarpBox::load<TPB>(ts), SS, sx, sy, sz);
+  NearMask<NP> nm{};
 #pragma unroll 1
   for (int j = 0; j < SEG; ++j) {
     const typename L::Src src = L::load(SS + j * V);
@@ -493,37 +573,36 @@ __device__ __noinline__ LaneAcc<NP> exact_segment(
       pair_d(tg.t[p], src.nx, src.ny, src.nz, dx[p], dy[p], dz[p], r2[p]);
       any |= (r2[p].x < tg.t[p].rc2.x) | (r2[p].y < tg.t[p].rc2.y);
     }
-    if (__any_sync(FULL, any)) {
+    if (((near_src >> j) & 1u) && __any_sync(FULL, any)) {
       const float4 yl = kFresh ? __ldcg(ylo + j) : ylo[j];
-      unsigned near_bits = 0;
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
-        const float4 hx = ts[(p * TGT_SLOTS) * TPB32], hy = ts[(p * TGT_SLOTS + 1) * TPB32],
-                     hz = ts[(p * TGT_SLOTS + 2) * TPB32];
+        const float4 hx = ts[(p * TGT_SLOTS) * TPB], hy = ts[(p * TGT_SLOTS + 1) * TPB],
+                     hz = ts[(p * TGT_SLOTS + 2) * TPB];
         const float2 wd = make_float2(hs * tg.t[p].idl.x > WIDE_FRAME ? 1.f : 0.f,
                                       hs * tg.t[p].idl.y > WIDE_FRAME ? 1.f : 0.f);
-        near_bits |= pair_general<L>(
-                         src, tg.t[p], dx[p], dy[p], dz[p], r2[p], acc.u[p], rho_lo, rho_hi,
-                         mul2(wd, sub2(shift_residual2(lo2(hx), hi2(hx), sx, tg.t[p].x),
-                                       make_float2(yl.x, yl.x))),
-                         mul2(wd, sub2(shift_residual2(lo2(hy), hi2(hy), sy, tg.t[p].y),
-                                       make_float2(yl.y, yl.y))),
-                         mul2(wd, sub2(shift_residual2(lo2(hz), hi2(hz), sz, tg.t[p].z),
-                                       make_float2(yl.z, yl.z))))
-                     << (2 * p);
+        pair_general<L>(
+            src, tg.t[p], dx[p], dy[p], dz[p], r2[p], acc.u[p], 1u << j, nm.m[2 * p],
+            nm.m[2 * p + 1],
+            mul2(wd, sub2(shift_residual2(lo2(hx), hi2(hx), sx, tg.t[p].x),
+                          make_float2(yl.x, yl.x))),
+            mul2(wd, sub2(shift_residual2(lo2(hy), hi2(hy), sy, tg.t[p].y),
+                          make_float2(yl.y, yl.y))),
+            mul2(wd, sub2(shift_residual2(lo2(hz), hi2(hz), sz, tg.t[p].z),
+                          make_float2(yl.z, yl.z))));
       }
-      near_append_warp<NP, kFresh>(near_bits, lane, group, orig + j, near_cnt, near_idx, flags);
     } else {
 #pragma unroll
       for (int p = 0; p < NP; ++p) L::far(src, dx[p], dy[p], dz[p], r2[p], acc.u[p]);
     }
   }
+  near_append_warp<NP, kFresh>(nm, group, orig, near_cnt, near_idx, flags);
   return acc;
 }
 
 // Shared memory of a pair item: the source stages; the per-thread target
 // state (TGT_SLOTS float4 per f32x2 pair: (hi, lo) of x, y, z, then
-// (1/delta, rho_c^2 delta^2), (rho_T^2 delta^2, -)), read once per segment;
+// (1/delta, rho_c^2 delta^2), (rho_T^2 delta^2, the warp's box), read once per segment;
 // and, for one pair per lane, the compensated accumulators. With one pair per
 // lane three CTAs share an SM, so that configuration runs one stage fewer.
 template <class L>
@@ -534,16 +613,16 @@ __host__ __device__ constexpr bool hilo_in_smem(int np) {
   // drop it to one CTA per SM, so it keeps them in registers)
   return np == 1 || (np == 2 && L::V == V_SL);
 }
-template <class L, int NP>
+template <class L, int NP, int TPB = TPB32>
 __host__ __device__ constexpr int pair_stages() {
-  return NP == 1 ? L::STAGES - 1 : L::STAGES;
+  return TPB < TPB32 ? 2 : NP == 1 ? L::STAGES - 1 : L::STAGES;
 }
 
-template <class L, int NP>
+template <class L, int NP, int TPB = TPB32>
 constexpr size_t pair_smem_bytes() {
-  return (size_t)pair_stages<L, NP>() * TILE * L::V * sizeof(float4) +
-         (size_t)NP * TGT_SLOTS * TPB32 * sizeof(float4) +
-         (hilo_in_smem<L>(NP) ? (size_t)NP * 6 * TPB32 * sizeof(float2) : 0);
+  return (size_t)pair_stages<L, NP, TPB>() * TILE * L::V * sizeof(float4) +
+         (size_t)NP * TGT_SLOTS * TPB * sizeof(float4) +
+         (hilo_in_smem<L>(NP) ? (size_t)NP * 6 * TPB * sizeof(float2) : 0);
 }
 
 // Shared-memory state of the source pipeline of one CTA.
@@ -563,14 +642,13 @@ struct PairArgs {
   const int* src_orig;
   const int* meta;
   const float4* tgtF;
-  const double4_32a* tgt64;
   int64_t M_pad;
   int n_chunks;
   double* part;
   int* near_cnt;       // per target group (64 * NP targets)
   unsigned* near_idx;  // per target group: NEAR_K * 64 * NP entries
   unsigned long long* flags;
-  float rho_lo, rho_hi;
+  float rt_ratio;  // near_radius2's ratio
   const float4* srcLo = nullptr;  // double layer: residuals of the packed positions
 };
 
@@ -622,28 +700,27 @@ __device__ __forceinline__ TileRange chunk_tiles(const PairArgs& a, int ch) {
   return TileRange{k0, k1 - k0, ch};
 }
 
-// One work item: target block tb (TPB32 * 2 * NP sorted targets) against
+// One work item: target block tb (TPB * 2 * NP sorted targets) against
 // the source tiles tl. Writes the block's partials (target t at
 // tl.out(a, t)); returns false if a bounded wait expired (the flag is set,
 // nothing is written).
 // kFresh: the evaluation's data is read with fresh loads (ld.global.cg), for
 // the server's persistent kernel.
-template <class L, int NP, bool kFresh = false, class TL>
+template <class L, int NP, int TPB = TPB32, bool kFresh = false, class TL>
 __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& tl, float4* sm,
-                                          PipeSmem<pair_stages<L, NP>()>& ps) {
+                                          PipeSmem<pair_stages<L, NP, TPB>()>& ps) {
   constexpr int V = L::V;
-  constexpr int STAGES = pair_stages<L, NP>();
-  constexpr int WARPS = TPB32 / 32;
+  constexpr int STAGES = pair_stages<L, NP, TPB>();
+  constexpr int WARPS = TPB / 32;
   constexpr uint32_t SEG_BYTES = SEG * V * sizeof(float4);
   const float4* __restrict__ srcF = a.srcF;
   const float4* __restrict__ segbox = a.segbox;
   const int* __restrict__ src_orig = a.src_orig;
   const float4* __restrict__ tgtF = a.tgtF;
-  const double4_32a* __restrict__ tgt64 = a.tgt64;
   int* __restrict__ near_cnt = a.near_cnt;
   unsigned* __restrict__ near_idx = a.near_idx;
   unsigned long long* __restrict__ flags = a.flags;
-  const float rho_lo = a.rho_lo, rho_hi = a.rho_hi;
+  const float rt_ratio = a.rt_ratio;
   uint64_t* full = ps.full;
   int* rel = ps.rel;
   int* issued = ps.issued;
@@ -652,10 +729,10 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
   const int n_it = tl.n;
 
   // ---- targets of this lane: pair p holds targets (base + 64p + lane, base + 64p + 32 + lane)
-  const int64_t wbase = (int64_t)tb * (TPB32 * 2 * NP) + wid * (64 * NP) + lane;
+  const int64_t wbase = (int64_t)tb * (TPB * 2 * NP) + wid * (64 * NP) + lane;
   // this warp's target group (its near-pair list)
-  const int64_t group = (int64_t)tb * (TPB32 / 32) + wid;
-  // per-thread target state: [(p * TGT_SLOTS + slot) * TPB32 + tid]
+  const int64_t group = (int64_t)tb * (TPB / 32) + wid;
+  // per-thread target state: [(p * TGT_SLOTS + slot) * TPB + tid]
   float4* const ts = sm + STAGES * TILE * V + tid;
   Tgt2 T[NP];
   float blo[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, bhi[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
@@ -675,8 +752,12 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
         rc2max = fmaxf(rc2max, b[h].x);
       }
     }
-    ts[(p * TGT_SLOTS + 3) * TPB32] = make_float4(a[0].w, a[1].w, b[0].x, b[1].x);
-    ts[(p * TGT_SLOTS + 4) * TPB32] = make_float4(b[0].y, b[1].y, 0.f, 0.f);
+    ts[(p * TGT_SLOTS) * TPB] = make_float4(a[0].x, a[1].x, b[0].y, b[1].y);
+    ts[(p * TGT_SLOTS + 1) * TPB] = make_float4(a[0].y, a[1].y, b[0].z, b[1].z);
+    ts[(p * TGT_SLOTS + 2) * TPB] = make_float4(a[0].z, a[1].z, b[0].w, b[1].w);
+    ts[(p * TGT_SLOTS + 3) * TPB] = make_float4(a[0].w, a[1].w, b[0].x, b[1].x);
+    ts[(p * TGT_SLOTS + 4) * TPB] = make_float4(near_radius2(b[0].x, rt_ratio),
+                                                  near_radius2(b[1].x, rt_ratio), 0.f, 0.f);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -688,20 +769,6 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
     rc2max = fmaxf(rc2max, __shfl_xor_sync(FULL, rc2max, o));
   }
   const bool warp_live = rc2max >= 0.f;
-  // FP32 (hi, lo) split of the targets' FP64 coordinates
-#pragma unroll
-  for (int p = 0; p < NP; ++p) {
-    const double4_32a x0 = kFresh ? ldcg4d(tgt64 + wbase + 64 * p) : tgt64[wbase + 64 * p],
-                      x1 = kFresh ? ldcg4d(tgt64 + wbase + 64 * p + 32)
-                                  : tgt64[wbase + 64 * p + 32];
-    const double a0[3] = {x0.x, x0.y, x0.z}, a1[3] = {x1.x, x1.y, x1.z};
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float h0 = (float)a0[c], h1 = (float)a1[c];
-      ts[(p * TGT_SLOTS + c) * TPB32] =
-          make_float4(h0, h1, (float)(a0[c] - (double)h0), (float)(a1[c] - (double)h1));
-    }
-  }
   float rc2test;
   {
     const float rc = sqrtf(fmaxf(rc2max, 0.f));
@@ -710,6 +777,10 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
                              fmaxf(fabsf(blo[2]), fabsf(bhi[2])));
     const float rm = rc * 1.00005f + box_margin(cmax, rc);
     rc2test = rm * rm;
+    // the warp's box, one component per lane (WarpBox)
+    const float v = lane < 3 ? (lane == 0 ? blo[0] : lane == 1 ? blo[1] : blo[2])
+                    : lane < 6 ? (lane == 3 ? bhi[0] : lane == 4 ? bhi[1] : bhi[2]) : rc2test;
+    reinterpret_cast<float*>(ts + 4 * TPB)[2] = v;
   }
 
   // Compensated accumulators (hi, lo): in shared memory, touched once per 128
@@ -717,14 +788,14 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
   constexpr bool kHiLoSmem = hilo_in_smem<L>(NP);
   float2 U[NP][3], HI[NP][3], LO[NP][3];
   // [(p * 3 + c) * 2 + {0: hi, 1: lo}][thread]: one float2 column per thread
-  float2* acc = reinterpret_cast<float2*>(sm + STAGES * TILE * V + NP * TGT_SLOTS * TPB32);
+  float2* acc = reinterpret_cast<float2*>(sm + STAGES * TILE * V + NP * TGT_SLOTS * TPB);
 #pragma unroll
   for (int p = 0; p < NP; ++p)
 #pragma unroll
     for (int c = 0; c < 3; ++c) U[p][c] = HI[p][c] = LO[p][c] = make_float2(0.f, 0.f);
   if constexpr (kHiLoSmem) {
 #pragma unroll
-    for (int i = 0; i < NP * 6; ++i) acc[i * TPB32 + tid] = make_float2(0.f, 0.f);
+    for (int i = 0; i < NP * 6; ++i) acc[i * TPB + tid] = make_float2(0.f, 0.f);
   }
 
   // ---- source pipeline: no CTA-wide barrier inside the loop; the last warp
@@ -783,10 +854,13 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
         const float4 lo = kFresh ? __ldcg(segbox + 2 * (sg + lane)) : segbox[2 * (sg + lane)];
         const float4 hi =
             kFresh ? __ldcg(segbox + 2 * (sg + lane) + 1) : segbox[2 * (sg + lane) + 1];
-        const float dx = fmaxf(0.f, fmaxf(lo.x - bhi[0], blo[0] - hi.x));
-        const float dy = fmaxf(0.f, fmaxf(lo.y - bhi[1], blo[1] - hi.y));
-        const float dz = fmaxf(0.f, fmaxf(lo.z - bhi[2], blo[2] - hi.z));
-        nb = dx * dx + dy * dy + dz * dz < rc2test;
+        // one pair per lane: the box from shared memory leaves the far loop
+        // its registers (cell of 24,576 nodes 415 -> 401 us, 96,774 sources x
+        // 5,766 targets 494 -> 449 us); two pairs: from registers (the
+        // stresslet at 221,184 nodes 20.3 -> 19.8 ms)
+        WarpBox wb{{blo[0], blo[1], blo[2]}, {bhi[0], bhi[1], bhi[2]}, rc2test};
+        if constexpr (NP == 1) wb = WarpBox::load<TPB>(ts);
+        nb = wb.reaches(make_float3(lo.x, lo.y, lo.z), make_float3(hi.x, hi.y, hi.z));
         csx = frame_mid(lo.x, hi.x);
         csy = frame_mid(lo.y, hi.y);
         csz = frame_mid(lo.z, hi.z);
@@ -801,8 +875,8 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
                     sz = __shfl_sync(FULL, csz, s);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-          const float4 hx = ts[(p * TGT_SLOTS) * TPB32], hy = ts[(p * TGT_SLOTS + 1) * TPB32],
-                       hz = ts[(p * TGT_SLOTS + 2) * TPB32];
+          const float4 hx = ts[(p * TGT_SLOTS) * TPB], hy = ts[(p * TGT_SLOTS + 1) * TPB],
+                       hz = ts[(p * TGT_SLOTS + 2) * TPB];
           T[p].x = shift_to_segment2(lo2(hx), hi2(hx), sx);
           T[p].y = shift_to_segment2(lo2(hy), hi2(hy), sy);
           T[p].z = shift_to_segment2(lo2(hz), hi2(hz), sz);
@@ -820,13 +894,6 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
           }
         } else {
           const int* orig = src_orig + (size_t)src0 + s * SEG;
-#pragma unroll
-          for (int p = 0; p < NP; ++p) {
-            const float4 q = ts[(p * TGT_SLOTS + 3) * TPB32], r = ts[(p * TGT_SLOTS + 4) * TPB32];
-            T[p].idl = lo2(q);
-            T[p].rc2 = hi2(q);
-            T[p].rt2 = lo2(r);
-          }
           // Exact differences (L::kExactNear) where the segment is wide for a
           // target: its frame half extent above WIDE_FRAME target deltas, so
           // that FP32 rounding of |x - c| and |y - c| could swamp an O(r^2)
@@ -835,6 +902,8 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
           bool wide = false;
           const float hs = __shfl_sync(FULL, chs, s);
           if constexpr (L::kExactNear) {
+#pragma unroll
+            for (int p = 0; p < NP; ++p) T[p].template load_radii<TPB>(ts + p * TGT_SLOTS * TPB);
 #pragma unroll
             for (int p = 0; p < NP; ++p)
               wide |= (hs * T[p].idl.x > WIDE_FRAME) | (hs * T[p].idl.y > WIDE_FRAME);
@@ -849,8 +918,8 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
 #pragma unroll
               for (int c = 0; c < 3; ++c) acc.u[p][c] = U[p][c];
             }
-            acc = general_segment<L, NP, kFresh>(acc, tg, SS, orig, group, near_cnt, near_idx, flags,
-                                         rho_lo, rho_hi);
+            acc = general_segment<L, NP, TPB, kFresh>(acc, tg, ts, sx, sy, sz, SS, orig, group, near_cnt,
+                                                 near_idx, flags);
 #pragma unroll
             for (int p = 0; p < NP; ++p)
 #pragma unroll
@@ -864,9 +933,9 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
 #pragma unroll
               for (int c = 0; c < 3; ++c) acc.u[p][c] = U[p][c];
             }
-            acc = exact_segment<L, NP, kFresh>(acc, tg, SS, a.srcLo + (size_t)src0 + s * SEG,
+            acc = exact_segment<L, NP, TPB, kFresh>(acc, tg, SS, a.srcLo + (size_t)src0 + s * SEG,
                                        orig, ts, sx, sy, sz, hs, group, near_cnt, near_idx,
-                                       flags, rho_lo, rho_hi);
+                                       flags);
 #pragma unroll
             for (int p = 0; p < NP; ++p)
 #pragma unroll
@@ -880,16 +949,16 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
             if constexpr (kHiLoSmem) {
 #pragma unroll
               for (int c = 0; c < 3; ++c) {
-                HI[p][c] = acc[((p * 3 + c) * 2) * TPB32 + tid];
-                LO[p][c] = acc[((p * 3 + c) * 2 + 1) * TPB32 + tid];
+                HI[p][c] = acc[((p * 3 + c) * 2) * TPB + tid];
+                LO[p][c] = acc[((p * 3 + c) * 2 + 1) * TPB + tid];
               }
             }
             two_sum_merge(U[p], HI[p], LO[p]);
             if constexpr (kHiLoSmem) {
 #pragma unroll
               for (int c = 0; c < 3; ++c) {
-                acc[((p * 3 + c) * 2) * TPB32 + tid] = HI[p][c];
-                acc[((p * 3 + c) * 2 + 1) * TPB32 + tid] = LO[p][c];
+                acc[((p * 3 + c) * 2) * TPB + tid] = HI[p][c];
+                acc[((p * 3 + c) * 2 + 1) * TPB + tid] = LO[p][c];
               }
             }
           }
@@ -933,11 +1002,11 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
       double* o = tl.out(a, t);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const float2 H2 = kHiLoSmem ? acc[((p * 3 + c) * 2) * TPB32 + tid] : HI[p][c];
-        const float2 L2 = kHiLoSmem ? acc[((p * 3 + c) * 2 + 1) * TPB32 + tid] : LO[p][c];
+        const float2 H2 = kHiLoSmem ? acc[((p * 3 + c) * 2) * TPB + tid] : HI[p][c];
+        const float2 L2 = kHiLoSmem ? acc[((p * 3 + c) * 2 + 1) * TPB + tid] : LO[p][c];
         const float hv = h ? H2.y : H2.x;
         const float lv = h ? L2.y : L2.x;
-        o[c] = (double)hv + (double)lv;
+        o[c] = widen(hv) + widen(lv);
       }
     }
   return true;
@@ -987,6 +1056,7 @@ struct OverflowArgs {
   const unsigned long long* flags;
   double* near_ovf;
   int group = 0;  // targets per group: 64 * (f32x2 pairs per lane) of the pair kernel
+  float rt_ratio = 0.f;  // near_radius2's ratio
 };
 
 struct FinishArgs {
@@ -1016,7 +1086,7 @@ __device__ __forceinline__ void rescan_target(const OverflowArgs& a, int64_t t, 
                                               double& u1, double& u2) {
   const int lane = threadIdx.x & 31;
   constexpr int V = L::V;
-  const float rt2 = a.tgtF[2 * t + 1].y;
+  const float rt2 = near_radius2(a.tgtF[2 * t + 1].x, a.rt_ratio);
   const double4_32a x = a.tgt64[t];
   const double invd = 1.0 / x.w;
   const float hx = (float)x.x, hy = (float)x.y, hz = (float)x.z;
@@ -1096,7 +1166,9 @@ __device__ __forceinline__ void sort_entries(unsigned* v, int n) {
 // Shared 32-bit words of one warp's near-sum scratch for groups of G targets:
 // the same in every kernel that finishes such groups, so that a target's sum
 // never depends on which kernel finished it.
-__host__ __device__ constexpr int near_warp_words(int G) { return G <= 64 ? 2048 : 3200; }
+// They include a warp's contributions (near_group's C), NEAR_C_WORDS.
+constexpr int NEAR_C_WORDS = 3 * 32 * 2;
+__host__ __device__ constexpr int near_warp_words(int G) { return G <= 64 ? 2176 : 3200; }
 
 // Barrier of a team of TEAM threads: one warp, or the whole CTA.
 template <int TEAM>
@@ -1105,84 +1177,163 @@ __device__ __forceinline__ void team_sync() {
   else __syncthreads();
 }
 
-// FP64 near sums of target group g (G = a.group targets) by a team of TEAM
+// Lanes that share a target's chunk partials in the finish: lane = 4 * sub +
+// (target of four), sub 0 .. 7. Each takes every eighth partial, and three
+// shuffles add the eight in a fixed order, the same in every kernel that
+// finishes targets.
+constexpr int FIN_SUBS = 8, FIN_TGTS = 32 / FIN_SUBS;
+__device__ __forceinline__ double fin_sum(double v) {
+#pragma unroll
+  for (int o = FIN_TGTS; o < 32; o *= 2) v += __shfl_xor_sync(FULL, v, o);
+  return v;
+}
+
+// v[0 .. n) (distinct) in ascending order, by one warp: each lane ranks its
+// value against the others; longer runs by one lane.
+__device__ __forceinline__ void sort_entries_warp(unsigned* v, int n) {
+  const int lane = threadIdx.x & 31;
+  if (n <= 32) {
+    const unsigned x = lane < n ? v[lane] : 0xffffffffu;
+    int r = 0;
+    for (int j = 0; j < n; ++j) r += __shfl_sync(FULL, x, j) < x ? 1 : 0;
+    __syncwarp();
+    if (lane < n) v[r] = x;
+  } else if (lane == 0) {
+    sort_entries(v, n);
+  }
+}
+
+// f(list[i]) for i = tid, tid + TEAM, .. < n, with four loads in flight.
+template <int TEAM, class F>
+__device__ __forceinline__ void for_entries(const unsigned* __restrict__ list, int n, int tid,
+                                            F f) {
+  for (int i = tid; i < n; i += 4 * TEAM) {
+    unsigned e[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i + q * TEAM < n) e[q] = list[i + q * TEAM];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i + q * TEAM < n) f(e[q]);
+  }
+}
+
+// FP64 near sums of targets [k0, k1) of group g (G targets) by a team of TEAM
 // threads (one warp, or a CTA of TEAM threads; tid = the thread's place in
-// it) with the shared words R[0 .. near_warp_words(G)); fin(t, n0, n1, n2)
-// then finishes target t (one thread per target). The group list is bucketed
-// by target in R, in passes over target ranges whose entries fit, and each
-// bucket sorted by source index: every target sums its near pairs in
-// ascending source order, whatever the order of the appends. The targets of
-// an overflowed group take their overflow rescan sums; a target with more
-// near pairs than R holds is rescanned here. Returns the near pairs this
-// thread counted.
-template <class L, int TEAM, class Fin>
+// it) with the shared words R[0 .. near_warp_words(G)) and TEAM double3 of
+// contributions C (see NEAR_C_WORDS); fin(t, valid, sub, n0, n1, n2) then
+// finishes target t: called by whole warps, FIN_SUBS lanes per target (all
+// with the target's sums), valid false on lanes without one.
+// The group list is bucketed by target in R, in passes over target ranges
+// whose entries fit, and each bucket sorted by source index. The pairs are then
+// evaluated one per lane whatever their target (a target has 0 to 30 or more,
+// so a lane per target would leave most of the FP64 pipe's issue to the
+// longest), a team's worth at a time through C; each target adds its own
+// contributions in ascending source order, whatever the order of the appends.
+// The targets of an overflowed group take their overflow rescan sums; a target
+// with more near pairs than R holds is rescanned here. Returns the near pairs
+// this thread counted.
+template <class L, int G, int TEAM, class Fin>
 __device__ __forceinline__ int near_group(const OverflowArgs& oa, const FinishArgs& a, int64_t g,
-                                          unsigned* R, int tid, Fin fin) {
-  const int G = a.group, CAP = NEAR_K * G, lane = tid & 31;
-  int* const cnt = reinterpret_cast<int*>(R);  // per target: count, then fill position
-  int* const beg = cnt + G;                    // per target: first entry (exclusive scan)
-  unsigned* const ent = R + 2 * G + 1;
-  const int EW = near_warp_words(G) - (2 * G + 1);
+                                          int k0, int k1, unsigned* R, double* C, int tid,
+                                          Fin fin) {
+  constexpr int CAP = NEAR_K * G;
+  constexpr unsigned SRC_MASK = (1u << NEAR_SRC_BITS) - 1u;
+  const int lane = tid & 31;
+  double* const sum = reinterpret_cast<double*>(R);  // [G][3] near sums
+  int* const cnt = reinterpret_cast<int*>(R + 6 * G);  // per target: count, then fill position
+  int* const beg = cnt + G;                            // per target: first entry (exclusive scan)
+  unsigned* const ent = R + 8 * G + 2;
+  constexpr int EW = near_warp_words(G) - NEAR_C_WORDS - (8 * G + 2);
   const int64_t tg0 = g * G;
   const int c = a.near_cnt[g];
+  const int sub = lane / FIN_TGTS, t8 = (tid >> 5) * FIN_TGTS + lane % FIN_TGTS;
+  constexpr int STEP = TEAM / FIN_SUBS;  // targets finished at a time
   if (c > CAP) {
-    for (int k = tid; k < G; k += TEAM) {
-      const int64_t t = tg0 + k;
-      fin(t, a.near_ovf[3 * t], a.near_ovf[3 * t + 1], a.near_ovf[3 * t + 2]);
+    for (int k = k0 + t8; k - t8 < k1; k += STEP) {
+      const bool valid = k < k1;
+      const int64_t t = tg0 + (valid ? k : k0);
+      fin(t, valid, sub, a.near_ovf[3 * t], a.near_ovf[3 * t + 1], a.near_ovf[3 * t + 2]);
     }
-    return tid == 0 ? c : 0;
+    return tid == 0 && k0 == 0 ? c : 0;
   }
   const unsigned* list = a.near_idx + (size_t)g * CAP;
   for (int k = tid; k < G; k += TEAM) cnt[k] = 0;
   team_sync<TEAM>();
-  for (int i = tid; i < c; i += TEAM) atomicAdd(&cnt[list[i] >> NEAR_SRC_BITS], 1);
+  for_entries<TEAM>(list, c, tid, [&](unsigned e) { atomicAdd(&cnt[e >> NEAR_SRC_BITS], 1); });
   team_sync<TEAM>();
   if (tid < 32) {
     int run = 0;
-    for (int k0 = 0; k0 < G; k0 += 32) {
-      const int v = cnt[k0 + lane];
+    for (int q = 0; q < G; q += 32) {
+      const int v = cnt[q + lane];
       int x = v;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int y = __shfl_up_sync(FULL, x, o);
         if (lane >= o) x += y;
       }
-      beg[k0 + lane] = run + x - v;
+      beg[q + lane] = run + x - v;
       run += __shfl_sync(FULL, x, 31);
     }
     if (lane == 0) beg[G] = run;
   }
   team_sync<TEAM>();
   int pairs = 0;
-  for (int ka = 0; ka < G;) {
+  for (int ka = k0; ka < k1;) {
     // the longest target range [ka, kb) whose entries fit (at least one target)
-    int lo = ka + 1, hi = G;
+    int lo = ka + 1, hi = k1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
       if (beg[mid] - beg[ka] <= EW) lo = mid;
       else hi = mid - 1;
     }
-    const int kb = lo, base = beg[ka];
-    if (beg[kb] - base <= EW) {
-      for (int k = ka + tid; k < kb; k += TEAM) cnt[k] = beg[k] - base;
-      team_sync<TEAM>();
-      for (int i = tid; i < c; i += TEAM) {
-        const unsigned e = list[i];
-        const int k = (int)(e >> NEAR_SRC_BITS);
-        if (k >= ka && k < kb) ent[atomicAdd(&cnt[k], 1)] = e & ((1u << NEAR_SRC_BITS) - 1u);
+    const int kb = lo, base = beg[ka], n = beg[kb] - base;
+    if (n <= EW) {
+      for (int k = ka + tid; k < kb; k += TEAM) {
+        cnt[k] = beg[k] - base;
+        sum[3 * k] = sum[3 * k + 1] = sum[3 * k + 2] = 0.0;
       }
       team_sync<TEAM>();
-      for (int k = ka + tid; k < kb; k += TEAM) {
-        const int64_t t = tg0 + k;
-        const int b0 = beg[k] - base, b1 = beg[k + 1] - base;
-        sort_entries(ent + b0, b1 - b0);
-        const double4_32a x = a.tgt64[t];
-        const double invd = 1.0 / x.w;
-        double n0 = 0, n1 = 0, n2 = 0;
-        for (int i = b0; i < b1; ++i)
-          Near64<L>::eval(x, a.xyz, a.w, a.dens, a.nrm, (int)ent[i], a.scale, invd, n0, n1, n2);
-        pairs += b1 - b0;
-        fin(t, n0, n1, n2);
+      for_entries<TEAM>(list, c, tid, [&](unsigned e) {
+        const int k = (int)(e >> NEAR_SRC_BITS);
+        if (k >= ka && k < kb) ent[atomicAdd(&cnt[k], 1)] = e;
+      });
+      team_sync<TEAM>();
+      for (int k = ka + (tid >> 5); k < kb; k += TEAM / 32)
+        sort_entries_warp(ent + beg[k] - base, beg[k + 1] - beg[k]);
+      team_sync<TEAM>();
+      for (int r = 0; r < n; r += TEAM) {
+        if (r + tid < n) {
+          const unsigned e = ent[r + tid];
+          const double4_32a x = a.tgt64[tg0 + (e >> NEAR_SRC_BITS)];
+          double v0 = 0, v1 = 0, v2 = 0;
+          Near64<L>::eval(x, a.xyz, a.w, a.dens, a.nrm, (int64_t)(e & SRC_MASK), a.scale,
+                          rcp_fp64(x.w), v0, v1, v2);
+          C[tid] = v0;
+          C[TEAM + tid] = v1;
+          C[2 * TEAM + tid] = v2;
+        }
+        team_sync<TEAM>();
+        // (target, component) of the targets with entries in this window
+        const int qa = 3 * (int)(ent[r] >> NEAR_SRC_BITS);
+        const int qb = 3 * (int)(ent[min(r + TEAM, n) - 1] >> NEAR_SRC_BITS) + 3;
+        for (int q = qa + tid; q < qb; q += TEAM) {
+          const int k = q / 3;
+          const int b0 = max(beg[k] - base, r), b1 = min(beg[k + 1] - base, r + TEAM);
+          if (b0 < b1) {
+            const double* v = C + (q - 3 * k) * TEAM - r;
+            double acc = sum[q];
+            for (int i = b0; i < b1; ++i) acc += v[i];
+            sum[q] = acc;
+          }
+        }
+        team_sync<TEAM>();
+      }
+      if (tid == 0) pairs += n;
+      for (int k = ka + t8; k - t8 < kb; k += STEP) {
+        const bool valid = k < kb;
+        const int q = valid ? k : ka;
+        fin(tg0 + q, valid, sub, sum[3 * q], sum[3 * q + 1], sum[3 * q + 2]);
       }
     } else if (tid < 32) {
       // target ka alone has more near pairs than R holds: the team's first
@@ -1190,10 +1341,8 @@ __device__ __forceinline__ int near_group(const OverflowArgs& oa, const FinishAr
       const int64_t t = tg0 + ka;
       double n0, n1, n2;
       rescan_target<L>(oa, t, n0, n1, n2);
-      if (lane == 0) {
-        pairs += beg[ka + 1] - base;
-        fin(t, n0, n1, n2);
-      }
+      if (lane == 0) pairs += n;
+      fin(t, lane % FIN_TGTS == 0, sub, n0, n1, n2);
     }
     team_sync<TEAM>();
     ka = kb;
@@ -1201,36 +1350,47 @@ __device__ __forceinline__ int near_group(const OverflowArgs& oa, const FinishAr
   return pairs;
 }
 
-// Near sums of targets t0 .. t0 + nt - 1 (whole groups) by the calling CTA:
-// warp w takes groups w, w + warps, ...; R holds near_warp_words(group) shared
-// words per warp.
-template <class L, class Fin>
+// Near sums of targets t0 .. t0 + nt - 1 (whole groups of G) by the calling
+// CTA: warp w takes groups w, w + warps, ...; R holds near_warp_words(G) shared
+// words per warp, the last NEAR_C_WORDS of them the warp's contributions.
+template <class L, int G, class Fin>
 __device__ __forceinline__ int near_groups(const OverflowArgs& oa, const FinishArgs& a,
                                            int64_t t0, int nt, unsigned* R, Fin fin) {
   const int wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int W = near_warp_words(a.group);
+  constexpr int W = near_warp_words(G);
+  static_assert(W % 2 == 0 && NEAR_C_WORDS % 2 == 0, "doubles at even words");
+  unsigned* const r = R + (size_t)wid * W;
   int pairs = 0;
-  for (int q = wid; q < nt / a.group; q += nw)
-    pairs += near_group<L, 32>(oa, a, t0 / a.group + q, R + (size_t)wid * W, threadIdx.x & 31,
-                               fin);
+  for (int q = wid; q < nt / G; q += nw)
+    pairs += near_group<L, G, 32>(oa, a, t0 / G + q, 0, G, r,
+                                  reinterpret_cast<double*>(r + W - NEAR_C_WORDS),
+                                  threadIdx.x & 31, fin);
   return pairs;
 }
 
-// Target t of a direct evaluation: its chunk partials in chunk order plus its
-// FP64 near sum, written at the target's original index.
-__device__ __forceinline__ void finish_merge(const FinishArgs& a, int64_t t, double n0, double n1,
-                                             double n2) {
+// Target t of a direct evaluation: its chunk partials plus its FP64 near sum,
+// written at the target's original index (see near_group's fin).
+__device__ __forceinline__ void finish_merge(const FinishArgs& a, int64_t t, bool valid, int sub,
+                                             double n0, double n1, double n2) {
   double u0 = 0, u1 = 0, u2 = 0;
-  for (int c = 0; c < a.n_chunks; ++c) {
-    const double* p = a.part + ((size_t)c * a.M_pad + t) * 3;
-    u0 += p[0];
-    u1 += p[1];
-    u2 += p[2];
+  if (valid) {
+#pragma unroll 8
+    for (int c = sub; c < a.n_chunks; c += FIN_SUBS) {
+      const double* p = a.part + ((size_t)c * a.M_pad + t) * 3;
+      u0 += p[0];
+      u1 += p[1];
+      u2 += p[2];
+    }
   }
-  const int64_t j = a.perm[t];
-  a.u[3 * j] = u0 + n0;
-  a.u[3 * j + 1] = u1 + n1;
-  a.u[3 * j + 2] = u2 + n2;
+  u0 = fin_sum(u0);
+  u1 = fin_sum(u1);
+  u2 = fin_sum(u2);
+  if (valid && sub == 0) {
+    const int64_t j = a.perm[t];
+    a.u[3 * j] = u0 + n0;
+    a.u[3 * j + 1] = u1 + n1;
+    a.u[3 * j + 2] = u2 + n2;
+  }
 }
 
 // Drop from L2, without writing them back, the 128-byte lines lying wholly
@@ -1245,21 +1405,26 @@ __device__ __forceinline__ void discard_l2(const void* begin, size_t bytes, int 
     asm volatile("discard.global.L2 [%0], 128;" ::"l"(q) : "memory");
 }
 
-// The scratch of targets t0 .. t0 + nt - 1 after their finish: their chunk
-// partials and near lists.
-__device__ __forceinline__ void discard_block_scratch(const FinishArgs& fa, int64_t t0, int nt,
-                                                      int tid, int n) {
+// The chunk partials of targets t0 .. t0 + nt - 1 after their finish.
+__device__ __forceinline__ void discard_block_partials(const FinishArgs& fa, int64_t t0, int nt,
+                                                       int tid, int n) {
   for (int c = 0; c < fa.n_chunks; ++c)
     discard_l2(fa.part + ((size_t)c * fa.M_pad + t0) * 3, (size_t)nt * 3 * sizeof(double), tid, n);
+}
+
+// ... and their near lists (whole groups).
+__device__ __forceinline__ void discard_block_scratch(const FinishArgs& fa, int64_t t0, int nt,
+                                                      int tid, int n) {
+  discard_block_partials(fa, t0, nt, tid, n);
   discard_l2(fa.near_idx + (size_t)t0 * NEAR_K, (size_t)nt * NEAR_K * sizeof(int), tid, n);
 }
 
 // Finish targets t0 .. t0 + nt - 1 (of M real ones) of a target block whose
 // chunks are all done: overflow rescans (if any list overflowed), FP64 near
 // sums and chunk merge, and the near-pair count. Run by a whole CTA, with
-// near_warp_words(group) free shared words per warp at sm; kept out of line
+// near_warp_words(G) free shared words per warp at sm; kept out of line
 // so that the pair loop's register allocation does not carry it.
-template <class L>
+template <class L, int G>
 __device__ __noinline__ void finish_block(const OverflowArgs& oa, const FinishArgs& fa, int64_t M,
                                           int64_t t0, int nt, unsigned* sm) {
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
@@ -1269,9 +1434,10 @@ __device__ __noinline__ void finish_block(const OverflowArgs& oa, const FinishAr
     __syncthreads();
     __threadfence_block();
   }
-  int cnt = near_groups<L>(oa, fa, t0, nt, sm, [&](int64_t t, double n0, double n1, double n2) {
-    if (t < M) finish_merge(fa, t, n0, n1, n2);
-  });
+  int cnt = near_groups<L, G>(
+      oa, fa, t0, nt, sm, [&](int64_t t, bool valid, int sub, double n0, double n1, double n2) {
+        finish_merge(fa, t, valid && t < M, sub, n0, n1, n2);
+      });
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
   if (lane == 0 && cnt) atomicAdd(fa.flags + FLAG_NEAR_PAIRS, (unsigned long long)cnt);
   __syncthreads();  // every read of the block's partials and near lists is done

@@ -74,14 +74,6 @@ __device__ __forceinline__ void far64(const double4_32a& G, const double4_32a& N
   }
 }
 
-// (double)w by integer instructions (an FP32-to-FP64 conversion would take the
-// FP64 pipe). Zero and subnormals come out as a nonzero value below 1.2e-38.
-__device__ __forceinline__ double widen(float w) {
-  const unsigned b = __float_as_uint(w);
-  const unsigned hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u);
-  return __hiloint2double((int)hi, (int)(b << 29));
-}
-
 // high words of y = 1 + rho^2 at the end of the smoothed range (rho = RHO_C64)
 // and at the end of the table
 static_assert(RHO_C64 == 7, "Y_NEAR_HI is the high word of 1 + 49");

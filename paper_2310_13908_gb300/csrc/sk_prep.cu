@@ -444,7 +444,7 @@ __global__ void k_pack_src64(const double* __restrict__ xyz, const double* __res
 
 __global__ void k_pack_tgt32(const double* __restrict__ xyz, const double* __restrict__ delta,
                              int64_t n_delta, const int* __restrict__ sorted, int64_t M,
-                             int64_t M_pad, double rho_T, double rho_c, float4* __restrict__ tgtF,
+                             int64_t M_pad, double rho_c, float4* __restrict__ tgtF,
                              double4_32a* __restrict__ tgt64, int* __restrict__ perm) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= M_pad) return;
@@ -452,10 +452,7 @@ __global__ void k_pack_tgt32(const double* __restrict__ xyz, const double* __res
   const int64_t j = sorted[real ? t : M - 1];
   const double x = xyz[3 * j], y = xyz[3 * j + 1], z = xyz[3 * j + 2];
   const double d = delta[n_delta == 1 ? 0 : j];
-  const double rc = rho_c * d, rt = rho_T * d;
-  tgtF[2 * t] = make_float4((float)x, (float)y, (float)z, (float)(1.0 / d));
-  tgtF[2 * t + 1] = real ? make_float4((float)(rc * rc), (float)(rt * rt), 0.f, 0.f)
-                         : make_float4(-1.f, -1.f, 0.f, 0.f);
+  write_tgt_record(tgtF + 2 * t, x, y, z, d, rho_c, real);
   tgt64[t] = make_double4_32a(x, y, z, d);
   perm[t] = real ? (int)j : -1;
 }
@@ -562,11 +559,10 @@ void launch_pack_sources64(int layer, const EvalBufs& b, double scale, cudaStrea
                                               b.N_pad, scale, b.src64, b.nrm64, b.segbox);
 }
 
-void launch_pack_targets32(const EvalBufs& b, int64_t n_delta, double rho_T, double rho_c,
-                           cudaStream_t st) {
+void launch_pack_targets32(const EvalBufs& b, int64_t n_delta, double rho_c, cudaStream_t st) {
   k_pack_tgt32<<<blocks_for(b.M_pad, 256), 256, 0, st>>>(b.tgt_xyz, b.delta, n_delta, b.tvals_a,
-                                                         b.M, b.M_pad, rho_T, rho_c, b.tgtF,
-                                                         b.tgt64, b.tgt_perm);
+                                                         b.M, b.M_pad, rho_c, b.tgtF, b.tgt64,
+                                                         b.tgt_perm);
 }
 
 void launch_pack_targets64(const EvalBufs& b, int64_t n_delta, cudaStream_t st) {

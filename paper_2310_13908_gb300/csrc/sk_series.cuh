@@ -21,42 +21,10 @@
 // time; kernels use them in Horner form in x = p^2 (no square root needed).
 #pragma once
 
+#include "sk_internal.h"
+#include "sk_near_factors.h"
+
 namespace sk {
-
-constexpr double INV_SQRT_PI = 0.56418958354775628695;  // 1/sqrt(pi)
-constexpr double PI_D = 3.14159265358979323846;
-
-__host__ __device__ constexpr double ecoef(int k) {
-  if (k < 0) return 0.0;
-  double v = 1.0;
-  for (int i = 1; i <= k; ++i) v /= (double)i;
-  return (k & 1) ? -v : v;
-}
-
-template <int N>
-struct Poly {
-  double c[N];
-};
-
-// which = 1: s1/p, 2: s2/p^3, 3: s3/p^5 (prefactor included)
-template <int WHICH, int N>
-__host__ __device__ constexpr Poly<N> series_coefs() {
-  Poly<N> P{};
-  for (int n = 0; n < N; ++n) {
-    double v = 0.0;
-    if (WHICH == 1)
-      v = (8.0 / 3.0) * INV_SQRT_PI * (2.0 * ecoef(n) - 4.0 * ecoef(n - 1) + ecoef(n - 2)) /
-          (2.0 * n + 1.0);
-    else if (WHICH == 2)
-      v = (16.0 / 3.0) * INV_SQRT_PI * (6.0 * ecoef(n) - 6.0 * ecoef(n - 1) + ecoef(n - 2)) /
-          (2.0 * n + 3.0);
-    else
-      v = (32.0 / 9.0) * INV_SQRT_PI * (12.0 * ecoef(n) - 8.0 * ecoef(n - 1) + ecoef(n - 2)) /
-          (2.0 * n + 5.0);
-    P.c[n] = v;
-  }
-  return P;
-}
 
 template <int WHICH, int N>
 __device__ __forceinline__ double horner(double x) {
@@ -68,17 +36,40 @@ __device__ __forceinline__ double horner(double x) {
 }
 
 // Series switch points in x = p^2. Relative truncation error of the three
-// series (exact rational arithmetic): 13 terms 1.3e-17 at x = 0.25 (p = 0.5,
-// the default rho_T of SK_FP32C); 16 terms 2.8e-20 at x = 0.36; 40 terms for
+// series (exact rational arithmetic): 16 terms 2.8e-20 at x = 0.36; 40 terms for
 // x < 4.84 (p < 2.2); beyond that the closed forms are used.
-constexpr double SERIES_X_TINY = 0.25;
 constexpr double SERIES_X_SHORT = 0.36;
 constexpr double SERIES_X_MAX = 4.84;
 
 template <int WHICH>
 __device__ __forceinline__ double series_factor(double x) {
-  if (x < SERIES_X_TINY) return horner<WHICH, 13>(x);
   return x < SERIES_X_SHORT ? horner<WHICH, 16>(x) : horner<WHICH, 40>(x);
+}
+
+static __device__ const NearFactors NEAR_FACTORS = near_factors();
+
+// Interval, offset from its middle (FP64 and FP32) of x in [0, NEAR_X_MAX).
+struct NearPoint {
+  double t;
+  float tf;
+  int i;
+};
+__device__ __forceinline__ NearPoint near_point(double x) {
+  constexpr double H = NEAR_X_MAX / NEAR_N;
+  const int i = min((int)(narrow(x) * (float)(1.0 / H)), NEAR_N - 1);
+  NearPoint p;
+  p.i = i;
+  p.t = x - widen(((float)i + 0.5f) * (float)H);
+  p.tf = narrow(p.t);
+  return p;
+}
+template <int WHICH>
+__device__ __forceinline__ double near_factor(const NearPoint& p) {
+  const auto& c = NEAR_FACTORS.c[WHICH - 1];
+  const auto& d = NEAR_FACTORS.t[WHICH - 1];
+  const float w = fmaf(fmaf(d[2][p.i], p.tf, d[1][p.i]), p.tf, d[0][p.i]) * p.tf;
+  return fma(fma(fma(fma(c[4][p.i] + widen(w), p.t, c[3][p.i]), p.t, c[2][p.i]), p.t, c[1][p.i]),
+             p.t, c[0][p.i]);
 }
 
 // Closed forms, FP64 (Sec. 3.4 for s1, s2; s3 as in the header).
@@ -102,11 +93,16 @@ __device__ __forceinline__ void sl_pair64(double dx, double dy, double dz, doubl
                                           double fz, double ws, double invd, double& u0,
                                           double& u1, double& u2) {
   const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+  const double i2 = invd * invd;
   const double x = r2 * invd * invd;
   double k1, k2;  // s1/r, s2/r^3
-  if (x < SERIES_X_MAX) {
+  if (x < NEAR_X_MAX) {
+    const NearPoint p = near_point(x);
+    k1 = near_factor<1>(p) * invd;
+    k2 = near_factor<2>(p) * (i2 * invd);
+  } else if (x < SERIES_X_MAX) {
     k1 = series_factor<1>(x) * invd;
-    k2 = series_factor<2>(x) * invd * invd * invd;
+    k2 = series_factor<2>(x) * (i2 * invd);
   } else {
     const double r = sqrt(r2);
     double s1, s2;
@@ -114,10 +110,10 @@ __device__ __forceinline__ void sl_pair64(double dx, double dy, double dz, doubl
     k1 = s1 / r;
     k2 = s2 / (r2 * r);
   }
-  const double fd = fma(fz, dz, fma(fy, dy, fx * dx));
-  u0 = fma(ws, fma(fx, k1, fd * dx * k2), u0);
-  u1 = fma(ws, fma(fy, k1, fd * dy * k2), u1);
-  u2 = fma(ws, fma(fz, k1, fd * dz * k2), u2);
+  const double b = ws * k2 * fma(fz, dz, fma(fy, dy, fx * dx)), a = ws * k1;
+  u0 = fma(b, dx, fma(a, fx, u0));
+  u1 = fma(b, dy, fma(a, fy, u1));
+  u2 = fma(b, dz, fma(a, fz, u2));
 }
 
 // One double-layer pair in FP64: u += ws (d.q)(d.n) d s3/r^5, ws = -6 w / (8 pi).
@@ -125,10 +121,12 @@ __device__ __forceinline__ void dl_pair64(double dx, double dy, double dz, doubl
                                           double qz, double nx, double ny, double nz, double ws,
                                           double invd, double& u0, double& u1, double& u2) {
   const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+  const double i2 = invd * invd;
   const double x = r2 * invd * invd;
   double k3;  // s3/r^5
-  if (x < SERIES_X_MAX) {
-    const double i2 = invd * invd;
+  if (x < NEAR_X_MAX) {
+    k3 = near_factor<3>(near_point(x)) * i2 * i2 * invd;
+  } else if (x < SERIES_X_MAX) {
     k3 = series_factor<3>(x) * i2 * i2 * invd;
   } else {
     const double r = sqrt(r2);

@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(TPB32, SERVE_MINB)
     // fresh loads: the arena block of an earlier request may have held other
     // data at these addresses while this kernel ran (a timeout sets the
     // request's flag)
-    pair_item<SLayer, SERVE_NP, true>(d.pa, tb, chunk_tiles<true>(d.pa, ch), sm, ps);
+    pair_item<SLayer, SERVE_NP, TPB32, true>(d.pa, tb, chunk_tiles<true>(d.pa, ch), sm, ps);
     __syncthreads();
     if (tid == 0) {
       __threadfence();
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(TPB32, SERVE_MINB)
       static_assert(pair_smem_bytes<SLayer, SERVE_NP>() / 4 >=
                         (size_t)(TPB32 / 32) * near_warp_words(64 * SERVE_NP),
                     "finish scratch");
-      finish_block<SLayer>(d.oa, d.fa, d.M, (int64_t)tb * SERVE_TGT_CTA, SERVE_TGT_CTA,
+      finish_block<SLayer, 64 * SERVE_NP>(d.oa, d.fa, d.M, (int64_t)tb * SERVE_TGT_CTA, SERVE_TGT_CTA,
                            reinterpret_cast<unsigned*>(sm));
       __syncthreads();
       if (tid == 0) {
@@ -396,15 +396,16 @@ void publish(sk_server* srv, int slot) {
   const EvalBufs& b = sl.b;
   const EvalShape& s = sl.req->shape;
   const double scale = layer_scale(s);
-  const float rho_lo = (float)srv->ctx->rho_T, rho_hi = 8.0f;
   SlotDesc d{};
-  d.pa = PairArgs{b.srcF, b.segbox, b.src_orig, b.meta, b.tgtF, b.tgt64, b.M_pad, b.n_chunks,
-                  b.part, b.near_cnt, b.near_idx, b.flags, rho_lo, rho_hi};
+  d.pa = PairArgs{b.srcF, b.segbox, b.src_orig, b.meta, b.tgtF, b.M_pad, b.n_chunks,
+                  b.part, b.near_cnt, b.near_idx, b.flags,
+                  near_ratio(srv->ctx->rho_T, srv->ctx->rho_c)};
   d.oa = OverflowArgs{b.srcF, b.segbox, b.src_orig, b.meta, b.tgtF, b.tgt64, b.near_cnt,
                       b.src_xyz, b.src_w, b.dens, b.nrm, scale, b.flags, b.near_ovf};
   d.fa = FinishArgs{b.tgt64, b.tgt_perm, b.M_pad, b.n_chunks, b.part, b.near_cnt, b.near_idx,
                     b.near_ovf, b.src_xyz, b.src_w, b.dens, b.nrm, scale, b.u, b.flags};
   d.oa.group = d.fa.group = 64 * SERVE_NP;
+  d.oa.rt_ratio = d.pa.rt_ratio;
   d.n_tb = (int)(b.M_pad / SERVE_TGT_CTA);
   d.tb_done = sl.tb_counters;
   d.tb_finished = sl.tb_counters + d.n_tb;
