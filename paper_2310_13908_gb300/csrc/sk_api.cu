@@ -118,6 +118,20 @@ void carve_eval_buffers(Bump& bp, const EvalShape& s, EvalBufs& b) {
     b.near_ovf = bp.take<double>((size_t)b.M_pad * 3);
   }
   b.flags = bp.take<unsigned long long>(N_FLAGS);
+  // Digit counts of the six-launch sorts. SK_FP32C: at the start of the near
+  // lists, which are written after the sorts (at least 384 KB; the counts take
+  // 2 KB per 256 points, at most 256 KB for the sources).
+  if (fp32) {
+    uint16_t* h = reinterpret_cast<uint16_t*>(b.near_idx);
+    const size_t nt = sort_mid_hist_words(s.M), ns = sort_mid_hist_words(s.N);
+    if ((nt + ns) * sizeof(uint16_t) <= (size_t)b.M_pad * NEAR_K * sizeof(unsigned)) {
+      b.tmid_hist = h;
+      b.mid_hist = h ? h + nt : nullptr;
+    }
+  } else {
+    b.tmid_hist = bp.take<uint16_t>(sort_mid_hist_words(s.M));
+    b.mid_hist = bp.take<uint16_t>(sort_mid_hist_words(s.N));
+  }
   // the target sort's own scratch last, so that the buffers above keep the
   // offsets they have without it
   if (s.split_sorts && s.N > 0) {
@@ -144,14 +158,8 @@ double layer_scale(const EvalShape& s) {
   return s.layer == LAYER_SL ? 1.0 / (8.0 * PI_CONST * s.mu) : -6.0 / (8.0 * PI_CONST);
 }
 
-__global__ void k_check_delta(const double* __restrict__ d, int64_t n,
-                              unsigned long long* __restrict__ flags) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n && !(d[i] > 0.0 && d[i] < INFINITY)) atomicExch(flags + FLAG_BAD_DELTA, 1ull);
-}
-
-// Preparation of one evaluation on `st`: clear the counters, check delta,
-// sort and pack sources and targets. With split sorts and a fork, the target
+// Preparation of one evaluation on `st`: clear the counters, sort and pack
+// sources and targets (the target pack checks delta). With split sorts and a fork, the target
 // sort and pack run on pf->aux beside the source sort and pack (the two touch
 // disjoint buffers; the result does not change), and `st` waits for them.
 // Returns the number of kernels launched.
@@ -159,16 +167,8 @@ int enqueue_prep(const EvalShape& s, const EvalBufs& b, double rho_T, double rho
                  cudaStream_t st, const PrepFork* pf) {
   const bool fp32 = s.precision == SK_FP32C;
   const double scale = layer_scale(s);
-  // bbox (2) + keys + 4 radix passes x 3 (hist, row scan, scatter), or the single-block sort
-  auto sort_launches = [&](int64_t n) { return n <= s.small_sort_points ? 1 : 3 + 4 * 3; };
   int launches = 0;
-  cudaMemsetAsync(b.flags, 0, N_FLAGS * sizeof(unsigned long long), st);
-  cudaMemsetAsync(b.meta, 0, N_META * sizeof(int), st);
-  if (fp32) {
-    cudaMemsetAsync(b.near_cnt, 0, (b.M_pad / NEAR_GROUP_MIN) * sizeof(int), st);
-    cudaMemsetAsync(b.tb_done, 0, (b.M_pad / 512 + 1) * sizeof(int), st);
-  }
-  k_check_delta<<<(unsigned)((s.n_delta + 255) / 256), 256, 0, st>>>(b.delta, s.n_delta, b.flags);
+  launch_clear(b, st);
   launches += 1;
   const bool fork = pf && pf->aux && s.split_sorts && s.N > 0;
   cudaStream_t tst = st;
@@ -178,20 +178,20 @@ int enqueue_prep(const EvalShape& s, const EvalBufs& b, double rho_T, double rho
     tst = pf->aux;
   }
   launch_sort_points(b.tgt_xyz, nullptr, s.M, b.tkeys_a, b.tkeys_b, b.tvals_a, b.tvals_b, b.thist,
-                     b.tbbox_part, b.tbbox, b.meta + META_SCRATCH, s.small_sort_points, tst);
-  launches += sort_launches(s.M);
+                     b.tbbox_part, b.tbbox, b.meta + META_SCRATCH, s.small_sort_points, b.tmid_hist, tst);
+  launches += sort_launches(s.M, s.small_sort_points, b.tmid_hist != nullptr);
   if (fp32)
     launch_pack_targets32(b, s.n_delta, rho_c, tst);
   else
     launch_pack_targets64(b, s.n_delta, tst);
   if (s.N > 0) {
     launch_sort_points(b.src_xyz, b.src_w, s.N, b.keys_a, b.keys_b, b.vals_a, b.vals_b, b.hist,
-                       b.bbox_part, b.bbox, b.meta + META_NS, s.small_sort_points, st);
+                       b.bbox_part, b.bbox, b.meta + META_NS, s.small_sort_points, b.mid_hist, st);
     if (fp32)
       launch_pack_sources32(s.layer, b, scale, st);
     else
       launch_pack_sources64(s.layer, b, scale, st);
-    launches += sort_launches(s.N) + 1;
+    launches += sort_launches(s.N, s.small_sort_points, b.mid_hist != nullptr) + 1;
   }
   if (fork) {
     cudaEventRecord(pf->join, pf->aux);

@@ -981,6 +981,7 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
     unsigned long long* sums = nullptr;  // [k][3] fixed-point coordinate sums
     unsigned int* cnt = nullptr;         // [k] points per cluster
     uint32_t *keys_a = nullptr, *keys_b = nullptr, *hist = nullptr;
+    uint16_t* mid_hist = nullptr;
     // FP32C
     int *vals_a = nullptr, *vals_b = nullptr, *meta = nullptr, *src_order = nullptr,
         *tgt_order = nullptr;
@@ -1023,6 +1024,8 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
     c.C32 = b.take<float4>(k);
     c.sums = b.take<unsigned long long>(3 * (size_t)k);
     c.cnt = b.take<unsigned int>(k);
+    c.mid_hist = b.take<uint16_t>(
+        std::max(sort_mid_hist_words(n_src), sort_mid_hist_words(n_tgt)));
     c.keys_a = b.take<uint32_t>(nsort);
     c.keys_b = b.take<uint32_t>(nsort);
     c.vals_a = b.take<int>(nsort);
@@ -1107,7 +1110,7 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
   };
   if (fp32) {
     launch_sort_points(X, W, n_src, cv.keys_a, cv.keys_b, cv.vals_a, cv.vals_b, cv.hist,
-                       cv.bbox_part, cv.bbox, cv.meta + META_SCRATCH, ctx->small_sort_points, st);
+                       cv.bbox_part, cv.bbox, cv.meta + META_SCRATCH, ctx->small_sort_points, cv.mid_hist, st);
     cudaMemcpyAsync(cv.src_order, cv.vals_a, n_src * sizeof(int), cudaMemcpyDeviceToDevice, st);
   }
   lists(lab, fp32 ? cv.src_order : nullptr, n_src, offs, count, list);
@@ -1116,7 +1119,7 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
   k_km_assign32<<<nblk(n_tgt), FMM_TPB, 0, st>>>(Y, nullptr, n_tgt, C, cv.C32, k, cv.tlab);
   if (fp32) {
     launch_sort_points(Y, nullptr, n_tgt, cv.keys_a, cv.keys_b, cv.vals_a, cv.vals_b, cv.hist,
-                       cv.bbox_part, cv.bbox, cv.meta + META_SCRATCH, ctx->small_sort_points, st);
+                       cv.bbox_part, cv.bbox, cv.meta + META_SCRATCH, ctx->small_sort_points, cv.mid_hist, st);
     cudaMemcpyAsync(cv.tgt_order, cv.vals_a, n_tgt * sizeof(int), cudaMemcpyDeviceToDevice, st);
   }
   lists(cv.tlab, fp32 ? cv.tgt_order : nullptr, n_tgt, cv.toffs, cv.tcount, cv.tlist);

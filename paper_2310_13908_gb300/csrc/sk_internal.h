@@ -219,6 +219,9 @@ struct EvalBufs {
   uint32_t* thist = nullptr;
   float* tbbox_part = nullptr;
   float* tbbox = nullptr;
+  // 16-bit digit counts of the six-launch sorts (sources, targets)
+  uint16_t* mid_hist = nullptr;
+  uint16_t* tmid_hist = nullptr;
   // prepared sources / targets
   int* meta = nullptr;
   int* src_orig = nullptr;        // packed source -> original index (-1: padding)
@@ -361,7 +364,12 @@ int enqueue_eval(const EvalShape& s, const EvalBufs& b, double rho_T, double rho
 void launch_sort_points(const double* xyz, const double* w, int64_t n, uint32_t* keys_a,
                         uint32_t* keys_b, int* vals_a, int* vals_b, uint32_t* hist,
                         float* bbox_part, float* bbox, int* count_out, int64_t small_max_points,
-                        cudaStream_t st);
+                        uint16_t* mid_hist, cudaStream_t st);
+// 16-bit words of mid_hist for n points (0: n has no use for it)
+size_t sort_mid_hist_words(int64_t n);
+// kernels launched by launch_sort_points (mid: with mid_hist)
+int sort_launches(int64_t n, int64_t small_max_points, bool mid);
+void launch_clear(const EvalBufs& b, cudaStream_t st);
 // Stable LSD radix sort of (key, value) pairs by the low `bits` bits of the
 // keys, 8 bits per pass, in the buffers of launch_sort_points (hist holds
 // 256 * sort_grid_blocks(n) + 256 words). Returns 0 when the sorted pairs are

@@ -10,6 +10,7 @@
 #include "sk_internal.h"
 
 #include <cfloat>
+#include <cmath>
 
 namespace sk {
 
@@ -64,9 +65,13 @@ __device__ void bbox_block(const double* __restrict__ xyz, const double* __restr
   if (threadIdx.x < 6) *out = s[threadIdx.x][0];
 }
 
+// clear: n_clear words to zero for a later launch.
 __global__ void k_bbox_partial(const double* __restrict__ xyz, const double* __restrict__ w,
-                               int64_t n, float* __restrict__ part) {
+                               int64_t n, float* __restrict__ part, uint32_t* __restrict__ clear,
+                               int n_clear) {
   __shared__ float s[6][RS_THREADS];
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_clear; i += gridDim.x * blockDim.x)
+    clear[i] = 0u;
   float v;
   bbox_block(xyz, w, n, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
              (int64_t)gridDim.x * blockDim.x, s, &v);
@@ -296,6 +301,163 @@ __global__ void __launch_bounds__(RS_THREADS)
                          base_d, wcnt);
 }
 
+// ---- the same order with six launches (up to RS_MID_MAX points) -------------
+// The launches of a mid-size sort are short, so their number is what counts:
+//   k_bbox_partial   partial boxes; clears the digit counts of passes 1 .. 3
+//   k_keys_hist      box from the partials, keys, digit counts of pass 0
+//   k_rs_pass (x 4)  per tile: offsets from all tiles' digit counts (each
+//                    block adds up the nblk <= 128 rows itself, coalesced),
+//                    stable scatter, and, at each key's new place, one count for
+//                    the next pass
+// against fifteen with a histogram and a row scan per pass. Two sorts of 24,576
+// points (targets and sources): 30 launches, 114 us one after another, now 12
+// and 81 us. Digit counts are 16-bit, [pass][tile][256] (a tile has at most 1024
+// keys).
+constexpr int64_t RS_MID_MAX = 131072;
+inline int rs_mid_items(int64_t n) { return n <= 32768 ? 1 : n <= 65536 ? 2 : 4; }
+constexpr int RS_PASSES = 4;
+
+template <int ITEMS>
+__global__ void __launch_bounds__(RS_THREADS)
+    k_keys_hist(const double* __restrict__ xyz, const double* __restrict__ w, int n,
+                const float* __restrict__ box_part, uint32_t* __restrict__ keys,
+                int* __restrict__ count, uint16_t* __restrict__ hist) {
+  __shared__ float box[6];
+  __shared__ uint32_t h[256];
+  const int tid = threadIdx.x, lane = tid & 31, c = tid >> 5;
+  h[tid] = 0;
+  if (c < 6) {
+    float v = c < 3 ? FLT_MAX : -FLT_MAX;
+    for (int b = lane; b < BBOX_BLOCKS; b += 32)
+      v = c < 3 ? fminf(v, box_part[b * 6 + c]) : fmaxf(v, box_part[b * 6 + c]);
+    for (int o = 16; o > 0; o >>= 1) {
+      const float y = __shfl_xor_sync(FULL, v, o);
+      v = c < 3 ? fminf(v, y) : fmaxf(v, y);
+    }
+    if (lane == 0) box[c] = v;
+  }
+  __syncthreads();
+  int act = 0;
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const int i = (blockIdx.x * ITEMS + r) * RS_THREADS + tid;
+    if (i < n) {
+      uint32_t key;
+      act += morton_key(xyz, w, i, box, &key) ? 1 : 0;
+      keys[i] = key;
+      atomicAdd(&h[key & 255u], 1u);
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) act += __shfl_xor_sync(FULL, act, o);
+  if (lane == 0 && act) atomicAdd(count, act);
+  __syncthreads();
+  hist[blockIdx.x * 256 + tid] = (uint16_t)h[tid];
+}
+
+// vin null: the values are the keys' places. kout null (last pass): keys are
+// not needed any more. hist_next null in the last pass.
+template <int ITEMS>
+__global__ void __launch_bounds__(RS_THREADS)
+    k_rs_pass(const uint32_t* __restrict__ kin, const int* __restrict__ vin,
+              uint32_t* __restrict__ kout, int* __restrict__ vout, int n, int shift,
+              const uint16_t* __restrict__ hist, uint32_t* __restrict__ hist_next) {
+  __shared__ uint32_t base_d[256];
+  __shared__ __align__(16) uint32_t wcnt[RS_THREADS / 32][256];
+  __shared__ __align__(16) uint32_t wbelow[RS_THREADS / 32][256];
+  __shared__ uint32_t warp_sums[RS_THREADS / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, blk = blockIdx.x;
+  // Digit counts over all tiles and over the tiles before this one. Warp w adds
+  // up rows w, w + 8, .., a lane eight digits of each (one 16-byte load): the
+  // at most 16 loads of a lane are in flight together.
+  {
+    uint32_t tot[8] = {}, bel[8] = {};
+#pragma unroll 8
+    for (int b = wid; b < (int)gridDim.x; b += RS_THREADS / 32) {
+      const uint4 v = *reinterpret_cast<const uint4*>(hist + b * 256 + 8 * lane);
+      const uint32_t q[4] = {v.x, v.y, v.z, v.w};
+      const bool before = b < blk;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t lo = q[c] & 0xffffu, hi = q[c] >> 16;
+        tot[2 * c] += lo;
+        tot[2 * c + 1] += hi;
+        bel[2 * c] += before ? lo : 0u;
+        bel[2 * c + 1] += before ? hi : 0u;
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      *reinterpret_cast<uint4*>(&wcnt[wid][8 * lane + 4 * c]) =
+          make_uint4(tot[4 * c], tot[4 * c + 1], tot[4 * c + 2], tot[4 * c + 3]);
+      *reinterpret_cast<uint4*>(&wbelow[wid][8 * lane + 4 * c]) =
+          make_uint4(bel[4 * c], bel[4 * c + 1], bel[4 * c + 2], bel[4 * c + 3]);
+    }
+  }
+  __syncthreads();
+  uint32_t below = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < RS_THREADS / 32; ++w) {
+    total += wcnt[w][tid];
+    below += wbelow[w][tid];
+  }
+  uint32_t all;
+  base_d[tid] = block_scan_incl(total, warp_sums, &all) - total + below;
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    for (int w = 0; w < RS_THREADS / 32; ++w) wcnt[w][tid] = 0;
+    __syncthreads();
+    const int i = (blk * ITEMS + r) * RS_THREADS + tid;
+    const bool valid = i < n;
+    const uint32_t key = valid ? kin[i] : 0u;
+    const int val = valid ? (vin ? vin[i] : i) : 0;
+    const uint32_t dig = (key >> shift) & 255u;
+    const unsigned peers = __match_any_sync(FULL, valid ? dig : (256u + lane));
+    const unsigned rank = __popc(peers & lt);
+    if (valid && rank == 0) wcnt[wid][dig] = __popc(peers);
+    __syncthreads();
+    if (valid) {
+      uint32_t off = 0;
+      for (int w = 0; w < wid; ++w) off += wcnt[w][dig];
+      const uint32_t pos = base_d[dig] + off + rank;
+      if (kout) kout[pos] = key;
+      vout[pos] = val;
+      if (hist_next) {
+        const uint32_t at = pos / (RS_THREADS * ITEMS) * 256u + ((key >> (shift + 8)) & 255u);
+        atomicAdd(hist_next + (at >> 1), (at & 1u) ? 0x10000u : 1u);
+      }
+    }
+    if (r + 1 < ITEMS) {
+      __syncthreads();
+      uint32_t add = 0;
+      for (int w = 0; w < RS_THREADS / 32; ++w) add += wcnt[w][tid];
+      base_d[tid] += add;
+      __syncthreads();
+    }
+  }
+}
+
+template <int ITEMS>
+void sort_mid(const double* xyz, const double* w, int n, uint32_t* keys_a, uint32_t* keys_b,
+              int* vals_a, int* vals_b, uint16_t* hist, float* bbox_part, int* count_out,
+              cudaStream_t st) {
+  const int nblk = rs_tiles(n, ITEMS), row = nblk * 256;
+  k_bbox_partial<<<BBOX_BLOCKS, RS_THREADS, 0, st>>>(
+      xyz, w, n, bbox_part, reinterpret_cast<uint32_t*>(hist + row), (RS_PASSES - 1) * row / 2);
+  k_keys_hist<ITEMS><<<nblk, RS_THREADS, 0, st>>>(xyz, w, n, bbox_part, keys_a, count_out, hist);
+  uint32_t *ka = keys_a, *kb = keys_b;
+  int *va = nullptr, *vb = vals_b;  // pass 0 takes the places as values
+  for (int p = 0; p < RS_PASSES; ++p) {
+    const bool last = p == RS_PASSES - 1;
+    k_rs_pass<ITEMS><<<nblk, RS_THREADS, 0, st>>>(
+        ka, va, last ? nullptr : kb, vb, n, 8 * p, hist + p * row,
+        last ? nullptr : reinterpret_cast<uint32_t*>(hist + (p + 1) * row));
+    uint32_t* tk = ka; ka = kb; kb = tk;
+    va = vb;
+    vb = va == vals_b ? vals_a : vals_b;
+  }
+}
+
 // The whole ordering of a small point set in one block of RS_THREADS threads:
 // box, Morton keys and the four radix passes, tile by tile, with the same
 // device code as the multi-block launches, so the order is the same. Saves
@@ -445,13 +607,15 @@ __global__ void k_pack_src64(const double* __restrict__ xyz, const double* __res
 __global__ void k_pack_tgt32(const double* __restrict__ xyz, const double* __restrict__ delta,
                              int64_t n_delta, const int* __restrict__ sorted, int64_t M,
                              int64_t M_pad, double rho_c, float4* __restrict__ tgtF,
-                             double4_32a* __restrict__ tgt64, int* __restrict__ perm) {
+                             double4_32a* __restrict__ tgt64, int* __restrict__ perm,
+                             unsigned long long* __restrict__ flags) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= M_pad) return;
   const bool real = t < M;
   const int64_t j = sorted[real ? t : M - 1];
   const double x = xyz[3 * j], y = xyz[3 * j + 1], z = xyz[3 * j + 2];
   const double d = delta[n_delta == 1 ? 0 : j];
+  if (!(d > 0.0 && d < INFINITY)) atomicExch(flags + FLAG_BAD_DELTA, 1ull);
   write_tgt_record(tgtF + 2 * t, x, y, z, d, rho_c, real);
   tgt64[t] = make_double4_32a(x, y, z, d);
   perm[t] = real ? (int)j : -1;
@@ -459,15 +623,29 @@ __global__ void k_pack_tgt32(const double* __restrict__ xyz, const double* __res
 
 __global__ void k_pack_tgt64(const double* __restrict__ xyz, const double* __restrict__ delta,
                              int64_t n_delta, const int* __restrict__ sorted, int64_t M,
-                             int64_t M_pad, double4_32a* __restrict__ tgt64, int* __restrict__ perm) {
+                             int64_t M_pad, double4_32a* __restrict__ tgt64, int* __restrict__ perm,
+                             unsigned long long* __restrict__ flags) {
   const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= M_pad) return;
   const bool real = t < M;
   const int64_t j = sorted[real ? t : M - 1];
   const double d = delta[n_delta == 1 ? 0 : j];
+  if (!(d > 0.0 && d < INFINITY)) atomicExch(flags + FLAG_BAD_DELTA, 1ull);
   // padding targets get a negative delta: the pair kernel skips them
   tgt64[t] = make_double4_32a(xyz[3 * j], xyz[3 * j + 1], xyz[3 * j + 2], real ? d : -1.0);
   perm[t] = real ? (int)j : -1;
+}
+
+// Counters of one evaluation at zero: flags, meta, near-list counts, finished
+// chunks per target block (one launch instead of four memsets).
+__global__ void k_clear(unsigned long long* __restrict__ flags, int* __restrict__ meta,
+                        int* __restrict__ near_cnt, int n_near, int* __restrict__ tb_done,
+                        int n_tb) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < N_FLAGS) flags[i] = 0ull;
+  if (i < N_META) meta[i] = 0;
+  if (i < n_near) near_cnt[i] = 0;
+  if (i < n_tb) tb_done[i] = 0;
 }
 
 inline unsigned blocks_for(int64_t n, int tpb) { return (unsigned)((n + tpb - 1) / tpb); }
@@ -480,6 +658,14 @@ int sort_grid_blocks(int64_t n) {
   const int fine = rs_tiles(n < RS_FINE_MAX ? n : RS_FINE_MAX, 1);
   const int coarse = rs_tiles(n, RS_ITEMS);
   return fine > coarse ? fine : coarse;
+}
+
+// 16-bit words of launch_sort_points' mid_hist for n points (0: not used).
+size_t sort_mid_hist_words(int64_t n) {
+  return n > 0 && n <= RS_MID_MAX ? (size_t)RS_PASSES * 256 * rs_tiles(n, rs_mid_items(n)) : 0;
+}
+int sort_launches(int64_t n, int64_t small_max_points, bool mid) {
+  return n <= small_max_points ? 1 : mid && n <= RS_MID_MAX ? 2 + RS_PASSES : 3 + 4 * 3;
 }
 
 // One radix pass (8 bits at shift) of n keys in nblk tiles of ITEMS keys per thread.
@@ -501,7 +687,7 @@ static void rs_pass(const uint32_t* ka, const int* va, uint32_t* kb, int* vb, in
 void launch_sort_points(const double* xyz, const double* w, int64_t n, uint32_t* keys_a,
                         uint32_t* keys_b, int* vals_a, int* vals_b, uint32_t* hist,
                         float* bbox_part, float* bbox, int* count_out, int64_t small_max_points,
-                        cudaStream_t st) {
+                        uint16_t* mid_hist, cudaStream_t st) {
   if (n <= 0) return;
   // tiles of this point set (at most the sort_grid_blocks the buffers hold);
   // the stable order does not depend on the tiling or on the path
@@ -510,7 +696,17 @@ void launch_sort_points(const double* xyz, const double* w, int64_t n, uint32_t*
                                            count_out, rs_tiles(n, RS_ITEMS));
     return;  // four passes: the sorted data is in keys_a / vals_a
   }
-  k_bbox_partial<<<BBOX_BLOCKS, RS_THREADS, 0, st>>>(xyz, w, n, bbox_part);
+  if (mid_hist && n <= RS_MID_MAX) {
+    const int items = rs_mid_items(n);
+    if (items == 1)
+      sort_mid<1>(xyz, w, (int)n, keys_a, keys_b, vals_a, vals_b, mid_hist, bbox_part, count_out, st);
+    else if (items == 2)
+      sort_mid<2>(xyz, w, (int)n, keys_a, keys_b, vals_a, vals_b, mid_hist, bbox_part, count_out, st);
+    else
+      sort_mid<4>(xyz, w, (int)n, keys_a, keys_b, vals_a, vals_b, mid_hist, bbox_part, count_out, st);
+    return;  // the sorted values are in vals_a (the keys are not kept)
+  }
+  k_bbox_partial<<<BBOX_BLOCKS, RS_THREADS, 0, st>>>(xyz, w, n, bbox_part, nullptr, 0);
   k_bbox_final<<<1, 6 * 32, 0, st>>>(bbox_part, BBOX_BLOCKS, bbox);
   k_morton_keys<<<blocks_for(n, 256), 256, 0, st>>>(xyz, w, n, bbox, keys_a, vals_a, count_out);
   uint32_t *ka = keys_a, *kb = keys_b;
@@ -535,6 +731,13 @@ int launch_sort_pairs(uint32_t* keys_a, uint32_t* keys_b, int* vals_a, int* vals
     int* tv = va; va = vb; vb = tv;
   }
   return passes & 1;
+}
+
+void launch_clear(const EvalBufs& b, cudaStream_t st) {
+  const int n_near = b.near_cnt ? (int)(b.M_pad / NEAR_GROUP_MIN) : 0;
+  const int n_tb = b.tb_done ? (int)(b.M_pad / 512 + 1) : 0;
+  k_clear<<<blocks_for(n_near > 256 ? n_near : 256, 256), 256, 0, st>>>(
+      b.flags, b.meta, b.near_cnt, n_near, b.tb_done, n_tb);
 }
 
 void launch_pack_sources32(int layer, const EvalBufs& b, double scale, cudaStream_t st) {
@@ -562,12 +765,13 @@ void launch_pack_sources64(int layer, const EvalBufs& b, double scale, cudaStrea
 void launch_pack_targets32(const EvalBufs& b, int64_t n_delta, double rho_c, cudaStream_t st) {
   k_pack_tgt32<<<blocks_for(b.M_pad, 256), 256, 0, st>>>(b.tgt_xyz, b.delta, n_delta, b.tvals_a,
                                                          b.M, b.M_pad, rho_c, b.tgtF, b.tgt64,
-                                                         b.tgt_perm);
+                                                         b.tgt_perm, b.flags);
 }
 
 void launch_pack_targets64(const EvalBufs& b, int64_t n_delta, cudaStream_t st) {
   k_pack_tgt64<<<blocks_for(b.M_pad, 256), 256, 0, st>>>(b.tgt_xyz, b.delta, n_delta, b.tvals_a,
-                                                         b.M, b.M_pad, b.tgt64, b.tgt_perm);
+                                                         b.M, b.M_pad, b.tgt64, b.tgt_perm,
+                                                         b.flags);
 }
 
 }  // namespace sk
