@@ -186,22 +186,29 @@ constexpr int KM_SMEM_SUMS = 512;      // clusters whose sums a block gathers in
 // largest coordinate magnitude of point and centres, so every centre within
 // 2^-16 (m + S^2) of the FP32 minimum m is a candidate and the FP64 minimum is
 // always among them. A point with a single candidate takes it (the FP64
-// minimum then is that centre); the FP64 distances decide between several,
-// in a pass that only blocks holding such points run. -1 for a zero-weight
-// point. C32: FP32 centres (x, y, z, largest |coordinate|).
-__global__ void __launch_bounds__(FMM_TPB) k_km_assign32(const double* __restrict__ X,
-                                                         const double* __restrict__ w, int64_t N,
-                                                         const double* __restrict__ C,
-                                                         const float4* __restrict__ C32, int k,
-                                                         int* __restrict__ lab) {
-  __shared__ float4 sc[KM_SMEM_CENTRES];
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// minimum then is that centre); one with two compares the two FP64 distances;
+// three or more are decided in a pass over the centres that only blocks
+// holding such points run. -1 for a zero-weight point. C32: FP32 centres
+// (x, y, z, largest |coordinate|). Returned for point i of the calling thread;
+// (x, y, z) gets the point.
+struct KmPoint {
+  double x, y, z;
+};
+__device__ __forceinline__ double km_dist2(const KmPoint& p, const double* __restrict__ c) {
+  const double dx = p.x - c[0], dy = p.y - c[1], dz = p.z - c[2];
+  return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+}
+__device__ __forceinline__ int km_nearest(const double* __restrict__ X,
+                                          const double* __restrict__ w, int64_t N, int64_t i,
+                                          const double* __restrict__ C,
+                                          const float4* __restrict__ C32, int k, float4* sc,
+                                          KmPoint& pt) {
   const bool live = i < N && !(w && w[i] == 0.0);
   const int64_t ii = i < N ? i : N - 1;
-  const double x = X[3 * ii], y = X[3 * ii + 1], z = X[3 * ii + 2];
-  const float xf = (float)x, yf = (float)y, zf = (float)z;
-  float m1 = INFINITY, m2 = INFINITY, cmax = 0.f;  // smallest, second smallest
-  int j1 = 0;
+  pt = KmPoint{X[3 * ii], X[3 * ii + 1], X[3 * ii + 2]};
+  const float xf = (float)pt.x, yf = (float)pt.y, zf = (float)pt.z;
+  float m1 = INFINITY, m2 = INFINITY, m3 = INFINITY, cmax = 0.f;  // the three smallest
+  int j1 = 0, j2 = 0;
   for (int j0 = 0; j0 < k; j0 += KM_SMEM_CENTRES) {
     const int nj = min(KM_SMEM_CENTRES, k - j0);
     __syncthreads();
@@ -211,20 +218,23 @@ __global__ void __launch_bounds__(FMM_TPB) k_km_assign32(const double* __restric
       const float4 c = sc[j];
       const float dx = xf - c.x, dy = yf - c.y, dz = zf - c.z;
       const float d = dx * dx + dy * dy + dz * dz;
-      if (d < m1) {
-        m2 = m1;
-        m1 = d;
-        j1 = j0 + j;
-      } else {
-        m2 = fminf(m2, d);
-      }
+      const bool first = d < m1, second = d < m2;
+      m3 = second ? m2 : fminf(m3, d);
+      m2 = first ? m1 : fminf(m2, d);
+      j2 = first ? j1 : second ? j0 + j : j2;
+      m1 = fminf(m1, d);
+      j1 = first ? j0 + j : j1;
       cmax = fmaxf(cmax, c.w);
     }
   }
   const float S = fmaxf(fabsf(xf), fmaxf(fabsf(yf), fabsf(zf))) + cmax;
   const float lim = m1 + 1.52587890625e-05f * (m1 + S * S);  // 2^-16
-  const bool several = m2 <= lim;
+  const bool several = m3 <= lim;
   int bj = j1;
+  if (m2 <= lim && !several) {
+    const double d1 = km_dist2(pt, C + 3 * (int64_t)j1), d2 = km_dist2(pt, C + 3 * (int64_t)j2);
+    if (d2 < d1 || (d2 == d1 && j2 < j1)) bj = j2;
+  }
   if (__syncthreads_or(several)) {
     double best = INFINITY;
     for (int j0 = 0; j0 < k; j0 += KM_SMEM_CENTRES) {
@@ -240,9 +250,7 @@ __global__ void __launch_bounds__(FMM_TPB) k_km_assign32(const double* __restric
         const float fx = xf - c.x, fy = yf - c.y, fz = zf - c.z;
         if (fx * fx + fy * fy + fz * fz > lim) continue;
         const int jj = j0 + j;
-        const double dx = x - C[3 * jj], dy = y - C[3 * jj + 1], dz = z - C[3 * jj + 2];
-        const double d2 =
-            __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+        const double d2 = km_dist2(pt, C + 3 * (int64_t)jj);
         if (d2 < best) {
           best = d2;
           bj = jj;
@@ -250,7 +258,19 @@ __global__ void __launch_bounds__(FMM_TPB) k_km_assign32(const double* __restric
       }
     }
   }
-  if (i < N) lab[i] = live ? bj : -1;
+  return live ? bj : -1;
+}
+
+__global__ void __launch_bounds__(FMM_TPB) k_km_assign32(const double* __restrict__ X,
+                                                         const double* __restrict__ w, int64_t N,
+                                                         const double* __restrict__ C,
+                                                         const float4* __restrict__ C32, int k,
+                                                         int* __restrict__ lab) {
+  __shared__ float4 sc[KM_SMEM_CENTRES];
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  KmPoint pt;
+  const int l = km_nearest(X, w, N, i, C, C32, k, sc, pt);
+  if (i < N) lab[i] = l;
 }
 
 // FP32 copies of the centres, with their largest |coordinate| in .w.
@@ -316,18 +336,24 @@ __global__ void k_km_frame(const double* __restrict__ part, int nblk, double* __
   frame[4] = 1.0 / frame[3];
 }
 
-// Exact sums of each cluster's points: every coordinate rounded to a
+// One Lloyd step's assignment and the exact sums of each cluster's points: every coordinate rounded to a
 // multiple of the quantum q above the box corner (at most 2^34 quanta) and
 // added in 64-bit integers, which makes the sums independent of the order of
 // the additions; point counts likewise. A warp first adds up the quanta of
 // its lanes that share a cluster (consecutive points mostly do), so one lane
 // per cluster and warp adds them on; for k <= KM_SMEM_SUMS a block gathers
-// those in shared memory first.
-__global__ void __launch_bounds__(FMM_TPB) k_km_sums(const double* __restrict__ X,
-                                                     const int* __restrict__ lab, int64_t N,
+// those in shared memory first. (One launch: the labels of an inner step are
+// needed by nothing else, and the points are in registers. Assignment, two
+// memsets and sums took 26 + 9 us and four launches per step at 98,304 points
+// and 128 centres; now 27 us and, with the centres' update, two.)
+__global__ void __launch_bounds__(FMM_TPB) k_km_step(const double* __restrict__ X,
+                                                     const double* __restrict__ w, int64_t N,
+                                                     const double* __restrict__ C,
+                                                     const float4* __restrict__ C32,
                                                      const double* __restrict__ frame, int k,
                                                      unsigned long long* __restrict__ sums,
                                                      unsigned int* __restrict__ cnt) {
+  __shared__ float4 sc[KM_SMEM_CENTRES];
   __shared__ unsigned long long ss[KM_SMEM_SUMS][3];
   __shared__ unsigned int sn[KM_SMEM_SUMS];
   const bool local = k <= KM_SMEM_SUMS;
@@ -340,12 +366,14 @@ __global__ void __launch_bounds__(FMM_TPB) k_km_sums(const double* __restrict__ 
   }
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
-  const int l = i < N ? lab[i] : -1;
+  KmPoint pt;
+  const int l = km_nearest(X, w, N, i, C, C32, k, sc, pt);
   unsigned long long q[3] = {0ull, 0ull, 0ull};
   if (l >= 0) {
     const double inv = frame[4];
+    const double x[3] = {pt.x, pt.y, pt.z};
     for (int a = 0; a < 3; ++a)
-      q[a] = (unsigned long long)llrint(fmax(X[3 * i + a] - frame[a], 0.0) * inv);
+      q[a] = (unsigned long long)llrint(fmax(x[a] - frame[a], 0.0) * inv);
   }
   // lanes of the same cluster (points without one form their own group)
   const unsigned grp = __match_any_sync(0xffffffffu, l);
@@ -381,9 +409,10 @@ __global__ void __launch_bounds__(FMM_TPB) k_km_sums(const double* __restrict__ 
 }
 
 // Thread per cluster: the centre moves to the mean of its points (an empty
-// cluster keeps its centre); the FP32 copy is refreshed.
-__global__ void k_km_centres(const unsigned long long* __restrict__ sums,
-                             const unsigned int* __restrict__ cnt,
+// cluster keeps its centre); the FP32 copy is refreshed and the sums are
+// cleared for the next step.
+__global__ void k_km_centres(unsigned long long* __restrict__ sums,
+                             unsigned int* __restrict__ cnt,
                              const double* __restrict__ frame, int k, double* __restrict__ C,
                              float4* __restrict__ C32) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -391,6 +420,8 @@ __global__ void k_km_centres(const unsigned long long* __restrict__ sums,
   if (cnt[j] != 0u)
     for (int a = 0; a < 3; ++a)
       C[3 * j + a] = frame[a] + ((double)sums[3 * j + a] / (double)cnt[j]) * frame[3];
+  for (int a = 0; a < 3; ++a) sums[3 * j + a] = 0ull;
+  cnt[j] = 0u;
   const float x = (float)C[3 * j], y = (float)C[3 * j + 1], z = (float)C[3 * j + 2];
   C32[j] = make_float4(x, y, z, fmaxf(fabsf(x), fmaxf(fabsf(y), fabsf(z))));
 }
@@ -812,21 +843,27 @@ __global__ void k_fmm_pack_tgt(const double* __restrict__ Y, const double* __res
   perm[t] = real ? (int)j : -1;
 }
 
+// Threads per CTA of the FMM's pair kernel. A box's targets are padded to whole
+// blocks: blocks of 256 targets (128 threads, one pair per lane) instead of 512
+// leave less padding to work through (98,304 targets in 128 boxes: 17% against
+// 40%).
+constexpr int fmm_pair_threads(int np) { return np == 1 ? 128 : TPB32; }
+
 // One work item per CTA: (target block, first tile descriptor, tiles,
 // partial slot); the block's partials go to slot * TB.
-template <int NP, int MINB>
-__global__ void __launch_bounds__(TPB32, MINB)
+template <int NP, int TPB, int MINB>
+__global__ void __launch_bounds__(TPB, MINB)
     k_pair32_fmm(p32::PairArgs a, const int4* __restrict__ items, const int2* __restrict__ desc) {
   extern __shared__ __align__(128) float4 sm[];
-  __shared__ p32::PipeSmem<p32::pair_stages<p32::SLayer, NP>()> ps;
+  __shared__ p32::PipeSmem<p32::pair_stages<p32::SLayer, NP, TPB>()> ps;
   if (threadIdx.x == 0) ps.initialized = 0;
-  constexpr int TB = TPB32 * 2 * NP;
+  constexpr int TB = TPB * 2 * NP;
   const int4 it = items[blockIdx.x];
-  p32::pair_item<p32::SLayer, NP>(
+  p32::pair_item<p32::SLayer, NP, TPB>(
       a, it.x, p32::TileList{desc + it.y, it.z, it.w, TB, (int64_t)it.x * TB}, sm, ps);
 }
 
-// FMM_FIN_PARTS CTAs per target group of G targets: each target's item partials
+// FMM_FIN_PARTS CTAs per target group of G targets (as k_finish32): each target's item partials
 // plus its FP64 near sum (the near-sum scratch in dynamic shared memory); u at
 // the target's original index.
 constexpr int FMM_FIN_PARTS = 2, FMM_FIN_THREADS = 128;
@@ -869,11 +906,12 @@ __global__ void __launch_bounds__(FMM_FIN_THREADS)
 template <int NP>
 void launch_pair32_fmm(const p32::PairArgs& a, const int4* items, const int2* desc, int n_items,
                        cudaStream_t st) {
-  constexpr int MINB = NP == 2 ? PAIR32_MINB_NP2 : PAIR32_MINB_NP1;
-  const size_t smem = p32::pair_smem_bytes<p32::SLayer, NP>();
-  cudaFuncSetAttribute(k_pair32_fmm<NP, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)smem);
-  k_pair32_fmm<NP, MINB><<<(unsigned)n_items, TPB32, smem, st>>>(a, items, desc);
+  constexpr int TPB = fmm_pair_threads(NP);
+  constexpr int MINB = (NP == 2 ? PAIR32_MINB_NP2 : PAIR32_MINB_NP1) * (TPB32 / TPB);
+  const size_t smem = p32::pair_smem_bytes<p32::SLayer, NP, TPB>();
+  const auto kernel = k_pair32_fmm<NP, TPB, MINB>;
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  kernel<<<(unsigned)n_items, TPB, smem, st>>>(a, items, desc);
 }
 
 // k_overflow32 of the direct path, for the FMM's targets.
@@ -951,7 +989,7 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
   // FP32C layout: target blocks of tb targets; equivalent sources padded to
   // whole segments; the bounds below size the workspace before the plan
   const int np32 = pair32_np(n_tgt);
-  const int tb = TPB32 * 2 * np32;
+  const int tb = fmm_pair_threads(np32) * 2 * np32;
   const int eqp = (int)align_up((size_t)Np, SEG);
   const int64_t near_slots_max = (int64_t)align_up((size_t)n_src, TILE) + (int64_t)k * TILE;
   const int64_t src_slots_max = near_slots_max + (int64_t)k * eqp;
@@ -1086,11 +1124,11 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
   k_km_frame_part<<<frame_blocks, FMM_TPB, 0, st>>>(X, W, n_src, cv.frame_part);
   k_km_frame<<<1, 32, 0, st>>>(cv.frame_part, frame_blocks, cv.frame);
   k_km_centres32<<<nblk(k), FMM_TPB, 0, st>>>(C, k, cv.C32);
+  cudaMemsetAsync(cv.sums, 0, 3 * (size_t)k * sizeof(unsigned long long), st);
+  cudaMemsetAsync(cv.cnt, 0, (size_t)k * sizeof(unsigned int), st);
   for (int it = 0; it < lloyd_iters; ++it) {
-    k_km_assign32<<<nblk(n_src), FMM_TPB, 0, st>>>(X, W, n_src, C, cv.C32, k, lab);
-    cudaMemsetAsync(cv.sums, 0, 3 * (size_t)k * sizeof(unsigned long long), st);
-    cudaMemsetAsync(cv.cnt, 0, (size_t)k * sizeof(unsigned int), st);
-    k_km_sums<<<nblk(n_src), FMM_TPB, 0, st>>>(X, lab, n_src, cv.frame, k, cv.sums, cv.cnt);
+    k_km_step<<<nblk(n_src), FMM_TPB, 0, st>>>(X, W, n_src, C, cv.C32, cv.frame, k, cv.sums,
+                                               cv.cnt);
     k_km_centres<<<nblk(k), FMM_TPB, 0, st>>>(cv.sums, cv.cnt, cv.frame, k, C, cv.C32);
   }
   k_km_assign32<<<nblk(n_src), FMM_TPB, 0, st>>>(X, W, n_src, C, cv.C32, k, lab);
