@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(FMM_FIN_THREADS)
     k_fmm_finish32(p32::OverflowArgs oa, p32::FinishArgs fa, const int* __restrict__ item_first,
                    int tb) {
   extern __shared__ __align__(16) unsigned fsm[];
-  constexpr int KP = G / FMM_FIN_PARTS;
+  constexpr int KP = G / FMM_FIN_PARTS, SUBS = p32::fin_subs(G);
   const int k0 = (int)(blockIdx.x % FMM_FIN_PARTS) * KP;
   int cnt = p32::near_group<p32::SLayer, G, FMM_FIN_THREADS>(
       oa, fa, blockIdx.x / FMM_FIN_PARTS, k0, k0 + KP, fsm,
@@ -882,16 +882,16 @@ __global__ void __launch_bounds__(FMM_FIN_THREADS)
         double u0 = 0.0, u1 = 0.0, u2 = 0.0;
         if (j >= 0) {
           const int64_t b = t / tb, l = t - b * tb;
-          for (int it = item_first[b] + sub; it < item_first[b + 1]; it += p32::FIN_SUBS) {
+          for (int it = item_first[b] + sub; it < item_first[b + 1]; it += SUBS) {
             const double* p = fa.part + ((size_t)it * tb + l) * 3;
             u0 += p[0];
             u1 += p[1];
             u2 += p[2];
           }
         }
-        u0 = p32::fin_sum(u0);
-        u1 = p32::fin_sum(u1);
-        u2 = p32::fin_sum(u2);
+        u0 = p32::fin_sum<SUBS>(u0);
+        u1 = p32::fin_sum<SUBS>(u1);
+        u2 = p32::fin_sum<SUBS>(u2);
         if (j >= 0 && sub == 0) {
           fa.u[3 * j] = u0 + n0;
           fa.u[3 * j + 1] = u1 + n1;

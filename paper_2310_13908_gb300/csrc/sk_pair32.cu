@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finish32(OverflowArgs oa, Finis
   int cnt = near_group<L, G, FIN_THREADS>(
       oa, a, g, k0, k0 + KP, fsm, reinterpret_cast<double*>(fsm + near_warp_words(G)), threadIdx.x,
       [&](int64_t t, bool valid, int sub, double n0, double n1, double n2) {
-        finish_merge(a, t, valid && t < M, sub, n0, n1, n2);
+        finish_merge<fin_subs(G)>(a, t, valid && t < M, sub, n0, n1, n2);
       });
   // count near pairs: one atomic per warp
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);

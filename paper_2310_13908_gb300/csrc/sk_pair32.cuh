@@ -502,8 +502,10 @@ __device__ __noinline__ LaneAcc<NP> general_segment(LaneAcc<NP> acc, LaneTgt<NP>
       far_four<L, NP>(acc, tg, SS + g * V);
       continue;
     }
-    if constexpr (NP == 1) {
-      // two sources at a time: two independent chains per warp
+    if constexpr (NP == 1 && !kFresh) {
+      // two sources at a time: two independent chains per warp (the server's
+      // kernel, with three CTAs per SM, has no registers for them: 24 requests 28.5
+      // ms, with two 29.1)
 #pragma unroll 1
       for (int j = g; j < g + 4; j += 2) {
         typename L::Src src[2];
@@ -1177,14 +1179,17 @@ __device__ __forceinline__ void team_sync() {
   else __syncthreads();
 }
 
-// Lanes that share a target's chunk partials in the finish: lane = 4 * sub +
-// (target of four), sub 0 .. 7. Each takes every eighth partial, and three
-// shuffles add the eight in a fixed order, the same in every kernel that
-// finishes targets.
-constexpr int FIN_SUBS = 8, FIN_TGTS = 32 / FIN_SUBS;
+// Lanes that share a target's chunk partials in the finish of groups of G
+// targets: lane = sub * (32 / SUBS) + target, sub 0 .. SUBS - 1. Each takes every
+// SUBS-th partial, and shuffles add the lanes' sums in a fixed order, the same
+// in every kernel that finishes such groups. Eight lanes for the small grids of
+// G = 64, which are short of threads; two for G = 128, where the additions count
+// (two FP64 lanes per clock and SM).
+__host__ __device__ constexpr int fin_subs(int G) { return G <= 64 ? 8 : 2; }
+template <int SUBS>
 __device__ __forceinline__ double fin_sum(double v) {
 #pragma unroll
-  for (int o = FIN_TGTS; o < 32; o *= 2) v += __shfl_xor_sync(FULL, v, o);
+  for (int o = 32 / SUBS; o < 32; o *= 2) v += __shfl_xor_sync(FULL, v, o);
   return v;
 }
 
@@ -1222,7 +1227,7 @@ __device__ __forceinline__ void for_entries(const unsigned* __restrict__ list, i
 // threads (one warp, or a CTA of TEAM threads; tid = the thread's place in
 // it) with the shared words R[0 .. near_warp_words(G)) and TEAM double3 of
 // contributions C (see NEAR_C_WORDS); fin(t, valid, sub, n0, n1, n2) then
-// finishes target t: called by whole warps, FIN_SUBS lanes per target (all
+// finishes target t: called by whole warps, fin_subs(G) lanes per target (all
 // with the target's sums), valid false on lanes without one.
 // The group list is bucketed by target in R, in passes over target ranges
 // whose entries fit, and each bucket sorted by source index. The pairs are then
@@ -1247,8 +1252,9 @@ __device__ __forceinline__ int near_group(const OverflowArgs& oa, const FinishAr
   constexpr int EW = near_warp_words(G) - NEAR_C_WORDS - (8 * G + 2);
   const int64_t tg0 = g * G;
   const int c = a.near_cnt[g];
-  const int sub = lane / FIN_TGTS, t8 = (tid >> 5) * FIN_TGTS + lane % FIN_TGTS;
-  constexpr int STEP = TEAM / FIN_SUBS;  // targets finished at a time
+  constexpr int TGTS = 32 / fin_subs(G);
+  const int sub = lane / TGTS, t8 = (tid >> 5) * TGTS + lane % TGTS;
+  constexpr int STEP = TEAM / fin_subs(G);  // targets finished at a time
   if (c > CAP) {
     for (int k = k0 + t8; k - t8 < k1; k += STEP) {
       const bool valid = k < k1;
@@ -1342,7 +1348,7 @@ __device__ __forceinline__ int near_group(const OverflowArgs& oa, const FinishAr
       double n0, n1, n2;
       rescan_target<L>(oa, t, n0, n1, n2);
       if (lane == 0) pairs += n;
-      fin(t, lane % FIN_TGTS == 0, sub, n0, n1, n2);
+      fin(t, lane % TGTS == 0, sub, n0, n1, n2);
     }
     team_sync<TEAM>();
     ka = kb;
@@ -1370,21 +1376,22 @@ __device__ __forceinline__ int near_groups(const OverflowArgs& oa, const FinishA
 
 // Target t of a direct evaluation: its chunk partials plus its FP64 near sum,
 // written at the target's original index (see near_group's fin).
+template <int SUBS>
 __device__ __forceinline__ void finish_merge(const FinishArgs& a, int64_t t, bool valid, int sub,
                                              double n0, double n1, double n2) {
   double u0 = 0, u1 = 0, u2 = 0;
   if (valid) {
 #pragma unroll 8
-    for (int c = sub; c < a.n_chunks; c += FIN_SUBS) {
+    for (int c = sub; c < a.n_chunks; c += SUBS) {
       const double* p = a.part + ((size_t)c * a.M_pad + t) * 3;
       u0 += p[0];
       u1 += p[1];
       u2 += p[2];
     }
   }
-  u0 = fin_sum(u0);
-  u1 = fin_sum(u1);
-  u2 = fin_sum(u2);
+  u0 = fin_sum<SUBS>(u0);
+  u1 = fin_sum<SUBS>(u1);
+  u2 = fin_sum<SUBS>(u2);
   if (valid && sub == 0) {
     const int64_t j = a.perm[t];
     a.u[3 * j] = u0 + n0;
@@ -1436,7 +1443,7 @@ __device__ __noinline__ void finish_block(const OverflowArgs& oa, const FinishAr
   }
   int cnt = near_groups<L, G>(
       oa, fa, t0, nt, sm, [&](int64_t t, bool valid, int sub, double n0, double n1, double n2) {
-        finish_merge(fa, t, valid && t < M, sub, n0, n1, n2);
+        finish_merge<fin_subs(G)>(fa, t, valid && t < M, sub, n0, n1, n2);
       });
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(FULL, cnt, o);
   if (lane == 0 && cnt) atomicAdd(fa.flags + FLAG_NEAR_PAIRS, (unsigned long long)cnt);
