@@ -70,7 +70,7 @@ typedef struct sk_ctx sk_ctx;
  * caller's stream still orders all of the call's work. *out is set to NULL
  * on failure. The environment variable SK_SMALL_SORT_POINTS (an integer
  * 0..2^24, read here) sets the largest point set that is ordered by the
- * single-block sort (default 3072; 0: always the multi-block sort); results
+ * single-block sort (default 1024; 0: always the multi-block sort); results
  * do not depend on it. */
 int sk_create(sk_ctx** out, int device, size_t workspace_bytes);
 

@@ -97,7 +97,6 @@ void carve_eval_buffers(Bump& bp, const EvalShape& s, EvalBufs& b) {
   b.hist = bp.take<uint32_t>(256 * (size_t)b.sort_blocks + 256);  // + the 256 row totals
   b.bbox_part = bp.take<float>(128 * 6);
   b.bbox = bp.take<float>(8);
-  b.meta = bp.take<int>(N_META);
   b.src_orig = bp.take<int>(b.N_pad);
   if (fp32) {
     b.srcF = bp.take<float4>((size_t)b.N_pad * (dl ? V_DL : V_SL));
@@ -117,7 +116,8 @@ void carve_eval_buffers(Bump& bp, const EvalShape& s, EvalBufs& b) {
     b.near_idx = bp.take<unsigned>((size_t)b.M_pad * NEAR_K);
     b.near_ovf = bp.take<double>((size_t)b.M_pad * 3);
   }
-  b.flags = bp.take<unsigned long long>(N_FLAGS);
+  b.flags = bp.take<unsigned long long>(N_FLAGS + N_META / 2);
+  b.meta = b.flags ? reinterpret_cast<int*>(b.flags + N_FLAGS) : nullptr;
   // Digit counts of the six-launch sorts. SK_FP32C: at the start of the near
   // lists, which are written after the sorts (at least 384 KB; the counts take
   // 2 KB per 256 points, at most 256 KB for the sources).
@@ -210,7 +210,7 @@ int enqueue_eval(const EvalShape& s, const EvalBufs& b, double rho_T, double rho
   if (ev) cudaEventRecord(ev[1], st);
   if (fp32) {
     launch_pair32(s.layer, b, rho_T, rho_c, scale, st, ev ? ev[2] : nullptr);  // with the finish
-    launches += b.fuse_finish ? 1 : 3;
+    launches += b.fuse_finish ? 1 : 2;
   } else {
     launch_pair64(s.layer, b, scale, st);
     if (ev) cudaEventRecord(ev[2], st);
@@ -453,10 +453,9 @@ int eval_entry(sk_ctx* ctx, int layer, int precision, int mem, int64_t N, const 
       enqueue_eval(s, b, ctx->rho_T, ctx->rho_c, st, ctx->profile ? ctx->ev : nullptr, &pf);
   if (mem == SK_HOST)
     cudaMemcpyAsync(u_out, b.u, 3 * M * sizeof(double), cudaMemcpyDeviceToHost, st);
-  cudaMemcpyAsync(ctx->h_flags, b.flags, N_FLAGS * sizeof(unsigned long long),
+  cudaMemcpyAsync(ctx->h_flags, b.flags,
+                  N_FLAGS * sizeof(unsigned long long) + N_META * sizeof(int),
                   cudaMemcpyDeviceToHost, st);
-  cudaMemcpyAsync(ctx->h_flags + N_FLAGS, b.meta, N_META * sizeof(int), cudaMemcpyDeviceToHost,
-                  st);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(ctx, e, fn);
   ctx->last_stream = st;
   ctx->stats = sk_eval_stats{};

@@ -874,6 +874,7 @@ __global__ void __launch_bounds__(FMM_FIN_THREADS)
   extern __shared__ __align__(16) unsigned fsm[];
   constexpr int KP = G / FMM_FIN_PARTS, SUBS = p32::fin_subs(G);
   const int k0 = (int)(blockIdx.x % FMM_FIN_PARTS) * KP;
+  p32::overflow_targets<p32::SLayer, G>(oa, blockIdx.x / FMM_FIN_PARTS, k0, k0 + KP, fa.M_pad);
   int cnt = p32::near_group<p32::SLayer, G, FMM_FIN_THREADS>(
       oa, fa, blockIdx.x / FMM_FIN_PARTS, k0, k0 + KP, fsm,
       reinterpret_cast<double*>(fsm + p32::near_warp_words(G)), threadIdx.x,
@@ -912,14 +913,6 @@ void launch_pair32_fmm(const p32::PairArgs& a, const int4* items, const int2* de
   const auto kernel = k_pair32_fmm<NP, TPB, MINB>;
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   kernel<<<(unsigned)n_items, TPB, smem, st>>>(a, items, desc);
-}
-
-// k_overflow32 of the direct path, for the FMM's targets.
-__global__ void k_fmm_overflow32(p32::OverflowArgs a, int64_t M) {
-  if (a.flags[FLAG_OVERFLOW] == 0ull) return;
-  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  if (t >= M) return;
-  p32::overflow_target<p32::SLayer>(a, t);
 }
 
 }  // namespace
@@ -1311,7 +1304,6 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
                            cv.flags,  cv.near_ovf};
       oa.group = 64 * np32;
       oa.rt_ratio = a.rt_ratio;
-      k_fmm_overflow32<<<(unsigned)((m_slots * 32 + 255) / 256), 256, 0, st>>>(oa, m_slots);
       p32::FinishArgs fa{cv.tgt64, cv.perm, m_slots, 1, cv.part, cv.near_cnt, cv.near_idx,
                          cv.near_ovf, X, W, F, nullptr, scale, U, cv.flags};
       fa.group = 64 * np32;

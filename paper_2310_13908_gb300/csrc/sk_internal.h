@@ -223,7 +223,7 @@ struct EvalBufs {
   uint16_t* mid_hist = nullptr;
   uint16_t* tmid_hist = nullptr;
   // prepared sources / targets
-  int* meta = nullptr;
+  int* meta = nullptr;            // directly behind the flags (one copy reads both)
   int* src_orig = nullptr;        // packed source -> original index (-1: padding)
   float4* srcF = nullptr;         // FP32 packed sources
   float4* srcLo = nullptr;        // double layer, FP32C: residual (y - c) - fl32(y - c) per source
@@ -306,10 +306,10 @@ namespace sk {
 
 // Largest point set ordered by the single-block sort by default;
 // SK_SMALL_SORT_POINTS in the environment of sk_create overrides it per
-// context (0 turns it off). Measured: one block costs ~24 us more per extra
-// 1024-point tile than the fifteen multi-block launches, and saves ~30 us at
-// two tiles, so the break-even is near three tiles.
-constexpr int64_t SMALL_SORT_POINTS = 3072;
+// context (0 turns it off). Measured (single layer, nodes as sources and
+// targets, single block / six launches): 384 points 112 / 120 us, 1014 121 / 123,
+// 1176 135 / 123, 1944 145 / 127, 2904 172 / 133.
+constexpr int64_t SMALL_SORT_POINTS = 1024;
 
 // CTA size of the FP64 pair kernel for problems too small to fill the GPU
 // with TPB64-thread CTAs (TPL64 targets per lane in both)
@@ -327,7 +327,7 @@ struct EvalShape {
   const char* factors64 = nullptr;  // SK_FP64: the context's factor tables
   bool fuse_finish = false;  // FP32C: finish target blocks inside the pair kernel
   // point sets of at most this many points are ordered by one single-block
-  // kernel instead of fifteen launches (0: never)
+  // kernel instead of six launches (0: never)
   int64_t small_sort_points = SMALL_SORT_POINTS;
   // the target sort takes scratch of its own and runs beside the source sort
   // on a second stream (context evaluations, capsule steps, served requests;
@@ -385,7 +385,7 @@ int sort_grid_blocks(int64_t n);
 // launchers (sk_pair32.cu / sk_pair64.cu)
 // FP32C pair sums and the finish of every target block (overflow rescans,
 // FP64 near sums, chunk merge, output write): fused into the pair kernel when
-// b.fuse_finish, else two more launches. pair_end (optional) is recorded
+// b.fuse_finish, else one more launch. pair_end (optional) is recorded
 // after the pair kernel, before any finish launch.
 void launch_pair32(int layer, const EvalBufs& b, double rho_T, double rho_c, double scale,
                    cudaStream_t st, cudaEvent_t pair_end = nullptr);

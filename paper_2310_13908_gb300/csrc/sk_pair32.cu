@@ -47,14 +47,6 @@ __global__ void __launch_bounds__(TPB32, MINB)
   finish_block<L, 64 * NP>(oa, fa, M, (int64_t)tb * TB, TB, reinterpret_cast<unsigned*>(sm));
 }
 
-template <class L>
-__global__ void k_overflow32(OverflowArgs a, int64_t M) {
-  if (a.flags[FLAG_OVERFLOW] == 0ull) return;
-  const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  if (t >= M) return;
-  overflow_target<L>(a, t);
-}
-
 // Separate finish for grids too small to fuse it: FIN_PARTS CTAs per target
 // group of G targets, each with its share of the targets (and the whole list,
 // of which it keeps its own), the near-sum scratch in dynamic shared memory.
@@ -71,6 +63,7 @@ __global__ void __launch_bounds__(FIN_THREADS) k_finish32(OverflowArgs oa, Finis
   constexpr int KP = G / FIN_PARTS;
   const int64_t g = blockIdx.x / FIN_PARTS;
   const int k0 = (int)(blockIdx.x % FIN_PARTS) * KP;
+  overflow_targets<L, G>(oa, g, k0, k0 + KP, M);
   int cnt = near_group<L, G, FIN_THREADS>(
       oa, a, g, k0, k0 + KP, fsm, reinterpret_cast<double*>(fsm + near_warp_words(G)), threadIdx.x,
       [&](int64_t t, bool valid, int sub, double n0, double n1, double n2) {
@@ -117,7 +110,6 @@ void launch_pair32_t(const EvalBufs& b, float rt_ratio, double scale,
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
     k<<<grid * (TPB32 / TPB), TPB, smem1, st>>>(a);
     if (pair_end) cudaEventRecord(pair_end, st);
-    k_overflow32<L><<<(unsigned)((b.M * 32 + 255) / 256), 256, 0, st>>>(oa, b.M);
     constexpr int G = 64 * NP;
     const size_t fsmem = (size_t)near_warp_words(G) * sizeof(unsigned) + FIN_THREADS * 3 * sizeof(double);
     k_finish32<L, G><<<(unsigned)(b.M_pad / G * FIN_PARTS), FIN_THREADS, fsmem, st>>>(oa, fa, b.M);

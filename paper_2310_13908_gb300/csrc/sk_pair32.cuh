@@ -1127,9 +1127,6 @@ __device__ __forceinline__ void overflow_target(const OverflowArgs& a, int64_t t
   }
 }
 
-// Finish one sorted target: chunk partials in fixed order plus the FP64 near
-// sum (list sorted by source index, or the overflow rescan's sum); writes
-// u at the target's original index. Returns the target's near-pair count.
 // v[0 .. n) in ascending order, by one thread: insertion sort for short runs,
 // heapsort for long ones (a group list may hold thousands of one target's
 // entries).
@@ -1354,6 +1351,17 @@ __device__ __forceinline__ int near_group(const OverflowArgs& oa, const FinishAr
     ka = kb;
   }
   return pairs;
+}
+
+// Rescans of targets [k0, k1) of group g if its list overflowed, by the warps of
+// the calling CTA (a rare case: more than NEAR_K near pairs per target).
+template <class L, int G>
+__device__ __forceinline__ void overflow_targets(const OverflowArgs& oa, int64_t g, int k0, int k1,
+                                                 int64_t M) {
+  if (oa.near_cnt[g] <= NEAR_K * G) return;
+  for (int k = k0 + (threadIdx.x >> 5); k < k1; k += blockDim.x >> 5)
+    if (g * G + k < M) overflow_target<L>(oa, g * G + k);
+  __syncthreads();
 }
 
 // Near sums of targets t0 .. t0 + nt - 1 (whole groups of G) by the calling

@@ -489,9 +489,9 @@ void scheduler(sk_server* srv) {
           r->st.done_us = now_us(srv);
           cudaMemcpyAsync(r->h_u, sl.b.u, 3 * r->shape.M * sizeof(double), cudaMemcpyDeviceToHost,
                           srv->s_copy);
-          cudaMemcpyAsync(sl.h_flags, sl.b.flags, N_FLAGS * sizeof(unsigned long long),
-                          cudaMemcpyDeviceToHost, srv->s_copy);
-          cudaMemcpyAsync(sl.h_flags + PIN_META, sl.b.meta, N_META * sizeof(int),
+          static_assert(PIN_META == N_FLAGS, "meta lies directly behind the flags");
+          cudaMemcpyAsync(sl.h_flags, sl.b.flags,
+                          N_FLAGS * sizeof(unsigned long long) + N_META * sizeof(int),
                           cudaMemcpyDeviceToHost, srv->s_copy);
           cudaEventRecord(sl.copy_done, srv->s_copy);
           sl.state = SlotState::Copying;
