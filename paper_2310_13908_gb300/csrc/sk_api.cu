@@ -6,8 +6,6 @@
 #include <cstring>
 #include <new>
 
-#include <vector>
-
 #include "sk_decomp.h"
 #include "sk_factors64.h"
 #include "sk_internal.h"
@@ -34,12 +32,9 @@ struct DeviceGuard {
 // The FP64 factor tables (136 KB), built once per process; every context
 // keeps a device copy.
 const char* factor_tables() {
-  static const std::vector<char> t = [] {
-    std::vector<char> v(F64_TABLES_BYTES);
-    f64_build_tables(v.data());
-    return v;
-  }();
-  return t.data();
+  alignas(double) static char t[F64_TABLES_BYTES];
+  static const bool built = (f64_build_tables(t), true);
+  return built ? t : nullptr;
 }
 
 int fail(sk_ctx* ctx, int code, const char* fmt, const char* detail = "") {
@@ -118,19 +113,18 @@ void carve_eval_buffers(Bump& bp, const EvalShape& s, EvalBufs& b) {
   }
   b.flags = bp.take<unsigned long long>(N_FLAGS + N_META / 2);
   b.meta = b.flags ? reinterpret_cast<int*>(b.flags + N_FLAGS) : nullptr;
-  // Digit counts of the six-launch sorts. SK_FP32C: at the start of the near
-  // lists, which are written after the sorts (at least 384 KB; the counts take
-  // 2 KB per 256 points, at most 256 KB for the sources).
-  if (fp32) {
-    uint16_t* h = reinterpret_cast<uint16_t*>(b.near_idx);
+  // Digit counts of the multi-launch sorts (2 KB per 256 points, at most 256 KB
+  // each): in the near lists (SK_FP32C) or the partials (SK_FP64), which are
+  // written after the sorts, so that they add nothing to the workspace. A sort
+  // whose counts do not fit there takes the launches of larger sets.
+  {
+    uint16_t* h = fp32 ? reinterpret_cast<uint16_t*>(b.near_idx)
+                       : reinterpret_cast<uint16_t*>(b.part);
+    const size_t room = fp32 ? (size_t)b.M_pad * NEAR_K * sizeof(unsigned)
+                             : (size_t)s.n_chunks * b.M_pad * 3 * sizeof(double);
     const size_t nt = sort_mid_hist_words(s.M), ns = sort_mid_hist_words(s.N);
-    if ((nt + ns) * sizeof(uint16_t) <= (size_t)b.M_pad * NEAR_K * sizeof(unsigned)) {
-      b.tmid_hist = h;
-      b.mid_hist = h ? h + nt : nullptr;
-    }
-  } else {
-    b.tmid_hist = bp.take<uint16_t>(sort_mid_hist_words(s.M));
-    b.mid_hist = bp.take<uint16_t>(sort_mid_hist_words(s.N));
+    if (h && nt * sizeof(uint16_t) <= room) b.tmid_hist = h;
+    if (h && (nt + ns) * sizeof(uint16_t) <= room) b.mid_hist = h + nt;
   }
   // the target sort's own scratch last, so that the buffers above keep the
   // offsets they have without it
@@ -256,8 +250,9 @@ int sk_create(sk_ctx** out, int device, size_t workspace_bytes) {
       (e = cudaEventCreateWithFlags(&ctx->join_ev, cudaEventDisableTiming)) != cudaSuccess ||
       (e = cudaMallocHost(&ctx->h_flags, 256)) != cudaSuccess ||
       (e = cudaMalloc(&ctx->factors64, F64_TABLES_BYTES)) != cudaSuccess ||
-      (e = cudaMemcpy(ctx->factors64, factor_tables(), F64_TABLES_BYTES,
-                      cudaMemcpyHostToDevice)) != cudaSuccess) {
+      (e = cudaMemcpyAsync(ctx->factors64, factor_tables(), F64_TABLES_BYTES,
+                           cudaMemcpyHostToDevice, ctx->aux_stream)) != cudaSuccess ||
+      (e = cudaStreamSynchronize(ctx->aux_stream)) != cudaSuccess) {
     code = e == cudaErrorMemoryAllocation ? SK_ENOMEM : SK_ECUDA;
   } else if (workspace_bytes > 0) {
     if ((e = cudaMalloc(&ctx->ws, workspace_bytes)) != cudaSuccess)

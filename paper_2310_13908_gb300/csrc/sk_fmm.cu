@@ -336,8 +336,8 @@ __global__ void k_km_frame(const double* __restrict__ part, int nblk, double* __
   frame[4] = 1.0 / frame[3];
 }
 
-// One Lloyd step's assignment and the exact sums of each cluster's points: every coordinate rounded to a
-// multiple of the quantum q above the box corner (at most 2^34 quanta) and
+// One Lloyd step's assignment and the exact sums of each cluster's points:
+// every coordinate rounded to a multiple of the quantum q above the box corner (at most 2^34 quanta) and
 // added in 64-bit integers, which makes the sums independent of the order of
 // the additions; point counts likewise. A warp first adds up the quanta of
 // its lanes that share a cluster (consecutive points mostly do), so one lane
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(256) k_fmm_phi(const double* __restrict__ P1T,
 }
 
 // Neighbouring-cluster sources, packed cluster by cluster (each cluster's
-// points in Morton order, padded to whole tiles): the FP32 records of the
+// points in curve order, padded to whole tiles): the FP32 records of the
 // direct sum. Slot s belongs to cluster tile_cluster[s / TILE].
 __global__ void k_fmm_pack_near(const double* __restrict__ X, const double* __restrict__ w,
                                 const double* __restrict__ f, const int* __restrict__ list,
@@ -819,7 +819,7 @@ __global__ void k_fmm_pack_eq(const double* __restrict__ box, const double* __re
   write_sl_record(srcF + (base + s) * V_SL, x, y, z, g0, g1, g2);
 }
 
-// Targets box by box (each box's targets in Morton order, padded to whole
+// Targets box by box (each box's targets in curve order, padded to whole
 // target blocks): slot t is in block t / tb, which belongs to box
 // block_box[t / tb]. Padding slots repeat one of the box's targets and are
 // dead (negative thresholds, perm = -1).
@@ -863,8 +863,8 @@ __global__ void __launch_bounds__(TPB, MINB)
       a, it.x, p32::TileList{desc + it.y, it.z, it.w, TB, (int64_t)it.x * TB}, sm, ps);
 }
 
-// FMM_FIN_PARTS CTAs per target group of G targets (as k_finish32): each target's item partials
-// plus its FP64 near sum (the near-sum scratch in dynamic shared memory); u at
+// FMM_FIN_PARTS CTAs per target group of G targets (as k_finish32): each
+// target's item partials plus its FP64 near sum (the near-sum scratch in dynamic shared memory); u at
 // the target's original index.
 constexpr int FMM_FIN_PARTS = 2, FMM_FIN_THREADS = 128;
 template <int G>
@@ -1012,7 +1012,6 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
     unsigned long long* sums = nullptr;  // [k][3] fixed-point coordinate sums
     unsigned int* cnt = nullptr;         // [k] points per cluster
     uint32_t *keys_a = nullptr, *keys_b = nullptr, *hist = nullptr;
-    uint16_t* mid_hist = nullptr;
     // FP32C
     int *vals_a = nullptr, *vals_b = nullptr, *meta = nullptr, *src_order = nullptr,
         *tgt_order = nullptr;
@@ -1055,8 +1054,6 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
     c.C32 = b.take<float4>(k);
     c.sums = b.take<unsigned long long>(3 * (size_t)k);
     c.cnt = b.take<unsigned int>(k);
-    c.mid_hist = b.take<uint16_t>(
-        std::max(sort_mid_hist_words(n_src), sort_mid_hist_words(n_tgt)));
     c.keys_a = b.take<uint32_t>(nsort);
     c.keys_b = b.take<uint32_t>(nsort);
     c.vals_a = b.take<int>(nsort);
@@ -1125,7 +1122,7 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
     k_km_centres<<<nblk(k), FMM_TPB, 0, st>>>(cv.sums, cv.cnt, cv.frame, k, C, cv.C32);
   }
   k_km_assign32<<<nblk(n_src), FMM_TPB, 0, st>>>(X, W, n_src, C, cv.C32, k, lab);
-  // each cluster's points listed in index order (FP64) or Morton order (FP32C,
+  // each cluster's points listed in index order (FP64) or curve order (FP32C,
   // the order of the direct sum): a stable sort of the points by label
   int key_bits = 1;
   while ((1ll << key_bits) <= (long long)k) ++key_bits;  // keys 0 .. k
@@ -1141,7 +1138,8 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
   };
   if (fp32) {
     launch_sort_points(X, W, n_src, cv.keys_a, cv.keys_b, cv.vals_a, cv.vals_b, cv.hist,
-                       cv.bbox_part, cv.bbox, cv.meta + META_SCRATCH, ctx->small_sort_points, cv.mid_hist, st);
+                       cv.bbox_part, cv.bbox, cv.meta + META_SCRATCH, ctx->small_sort_points,
+                       reinterpret_cast<uint16_t*>(cv.srcF), st);  // srcF is packed later
     cudaMemcpyAsync(cv.src_order, cv.vals_a, n_src * sizeof(int), cudaMemcpyDeviceToDevice, st);
   }
   lists(lab, fp32 ? cv.src_order : nullptr, n_src, offs, count, list);
@@ -1150,7 +1148,8 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
   k_km_assign32<<<nblk(n_tgt), FMM_TPB, 0, st>>>(Y, nullptr, n_tgt, C, cv.C32, k, cv.tlab);
   if (fp32) {
     launch_sort_points(Y, nullptr, n_tgt, cv.keys_a, cv.keys_b, cv.vals_a, cv.vals_b, cv.hist,
-                       cv.bbox_part, cv.bbox, cv.meta + META_SCRATCH, ctx->small_sort_points, cv.mid_hist, st);
+                       cv.bbox_part, cv.bbox, cv.meta + META_SCRATCH, ctx->small_sort_points,
+                       reinterpret_cast<uint16_t*>(cv.near_idx), st);  // near_idx is written later
     cudaMemcpyAsync(cv.tgt_order, cv.vals_a, n_tgt * sizeof(int), cudaMemcpyDeviceToDevice, st);
   }
   lists(cv.tlab, fp32 ? cv.tgt_order : nullptr, n_tgt, cv.toffs, cv.tcount, cv.tlist);

@@ -219,7 +219,7 @@ struct EvalBufs {
   uint32_t* thist = nullptr;
   float* tbbox_part = nullptr;
   float* tbbox = nullptr;
-  // 16-bit digit counts of the six-launch sorts (sources, targets)
+  // 16-bit digit counts of the multi-launch sorts (sources, targets)
   uint16_t* mid_hist = nullptr;
   uint16_t* tmid_hist = nullptr;
   // prepared sources / targets
@@ -307,7 +307,7 @@ namespace sk {
 // Largest point set ordered by the single-block sort by default;
 // SK_SMALL_SORT_POINTS in the environment of sk_create overrides it per
 // context (0 turns it off). Measured (single layer, nodes as sources and
-// targets, single block / six launches): 384 points 112 / 120 us, 1014 121 / 123,
+// targets, single block / six launches, now five): 384 points 112 / 120 us, 1014 121 / 123,
 // 1176 135 / 123, 1944 145 / 127, 2904 172 / 133.
 constexpr int64_t SMALL_SORT_POINTS = 1024;
 
@@ -327,7 +327,7 @@ struct EvalShape {
   const char* factors64 = nullptr;  // SK_FP64: the context's factor tables
   bool fuse_finish = false;  // FP32C: finish target blocks inside the pair kernel
   // point sets of at most this many points are ordered by one single-block
-  // kernel instead of six launches (0: never)
+  // kernel instead of five launches (0: never)
   int64_t small_sort_points = SMALL_SORT_POINTS;
   // the target sort takes scratch of its own and runs beside the source sort
   // on a second stream (context evaluations, capsule steps, served requests;

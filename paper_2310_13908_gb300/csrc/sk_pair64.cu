@@ -3,9 +3,9 @@
 // Same work decomposition as the FP32 kernels (sorted targets, chunks of
 // source tiles staged by bulk async copies, per-segment near/far test), all
 // arithmetic in FP64:
-//   rho >= 7          plain Stokeslet / stresslet (s_i = 1 to double precision)
-//   2.2 <= rho < 7    closed-form s_i with erf/exp (Sec. 3.4)
-//   rho < 2.2         power series of s_i / rho^k (sk_series.cuh), incl. r = 0
+//   rho >= 7   plain Stokeslet / stresslet (s_i = 1 to double precision)
+//   rho < 7    s_i / rho^k from a table of local polynomials in rho^2
+//              (sk_factors64.h), incl. r = 0
 // Two targets per lane; plain FP64 accumulation per chunk; the finish
 // kernel adds the chunks of a target in fixed order.
 #include <cfloat>
