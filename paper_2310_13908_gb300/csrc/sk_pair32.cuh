@@ -655,8 +655,8 @@ struct PairArgs {
 };
 
 // The source tiles of one work item: n tiles, each (first packed source,
-// segments of SEG sources, at most TILE_SEGS). With desc == nullptr they are
-// the full tiles k0 .. k0 + n - 1 of the packed array; a list serves work
+// segments of SEG sources, at most TILE_SEGS). Every step-th full tile of the
+// packed array (TileStride), or a list (TileList) for work
 // whose tiles are scattered (the FMM's neighbouring clusters and
 // equivalent sources).
 // out(a, t): where the item writes target t's partial. A list's item
@@ -675,31 +675,35 @@ struct TileList {
     return a.part + ((size_t)slot * tb + (size_t)(t - t_sub)) * 3;
   }
 };
-// A contiguous range of full tiles k0 .. k0 + n - 1 of source chunk ch
-// (known to be full at compile time, so the direct evaluation's loops keep
-// their fixed shape); partials at [ch][M_pad][3].
-struct TileRange {
+// The n full tiles ch, ch + step, .. of source chunk ch (known to be full at
+// compile time, so the direct evaluation's loops keep their fixed shape);
+// partials at [ch][M_pad][3].
+struct TileStride {
   static constexpr bool kFull = true;
-  int k0, n, ch;
+  int ch, step, n;
+  __device__ __forceinline__ int index(int it) const { return ch + it * step; }
   __device__ __forceinline__ int2 tile(int it) const {
-    return make_int2((k0 + it) * TILE, TILE_SEGS);
+    return make_int2(index(it) * TILE, TILE_SEGS);
   }
   __device__ __forceinline__ size_t first_segment(int it, int) const {
-    return (size_t)(k0 + it) * TILE_SEGS;
+    return (size_t)index(it) * TILE_SEGS;
   }
   __device__ __forceinline__ double* out(const PairArgs& a, int64_t t) const {
     return a.part + ((size_t)ch * a.M_pad + t) * 3;
   }
 };
 
-// Tiles of source chunk ch of a direct evaluation: an even split of the
-// padded sources into a.n_chunks contiguous ranges.
+// Tiles of source chunk ch of a direct evaluation: every a.n_chunks-th tile. The
+// tiles near a target block follow one another in the sorted order; dealt out
+// to all chunks, they make its CTAs equally long, where one or two contiguous
+// chunks with all of them ran several times as long as the rest and
+// idled the chip at the end of the launch. (Pair kernel, contiguous chunks / dealt
+// out: 96,774 sources x 5,766 targets 412 / 327 us; 135,168 x 221,184, stresslet,
+// 20.73 / 19.87 ms; 239,880 x 493,216 68.84 / 67.93 ms.)
 template <bool kFresh = false>
-__device__ __forceinline__ TileRange chunk_tiles(const PairArgs& a, int ch) {
+__device__ __forceinline__ TileStride chunk_tiles(const PairArgs& a, int ch) {
   const int n_tiles = (kFresh ? __ldcg(a.meta + META_NS_PAD) : a.meta[META_NS_PAD]) / TILE;
-  const int k0 = (int)((long long)ch * n_tiles / a.n_chunks);
-  const int k1 = (int)((long long)(ch + 1) * n_tiles / a.n_chunks);
-  return TileRange{k0, k1 - k0, ch};
+  return TileStride{ch, a.n_chunks, (n_tiles - ch + a.n_chunks - 1) / a.n_chunks};
 }
 
 // One work item: target block tb (TPB * 2 * NP sorted targets) against
@@ -819,7 +823,7 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
     for (int b = 0; b < STAGES; ++b)
       if (b < n_it) {
         if constexpr (TL::kFull) {
-          bulk_load(sm + b * TILE * V, srcF + (size_t)(tl.k0 + b) * TILE * V, TILE * V * 16u,
+          bulk_load(sm + b * TILE * V, srcF + (size_t)tl.index(b) * TILE * V, TILE * V * 16u,
                     &full[b]);
         } else {
           const int2 t = tl.tile(b);
@@ -832,7 +836,7 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
     // first packed source and segments of this tile
     int src0, nseg;
     if constexpr (TL::kFull) {
-      src0 = (tl.k0 + it) * TILE;
+      src0 = tl.index(it) * TILE;
       nseg = TILE_SEGS;
     } else {
       const int2 tile = tl.tile(it);
@@ -976,7 +980,7 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
         __threadfence_block();
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         if constexpr (TL::kFull) {
-          bulk_load(sm + buf * TILE * V, srcF + (size_t)(tl.k0 + it + STAGES) * TILE * V,
+          bulk_load(sm + buf * TILE * V, srcF + (size_t)tl.index(it + STAGES) * TILE * V,
                     TILE * V * 16u, &full[buf]);
         } else {
           const int2 t = tl.tile(it + STAGES);
