@@ -1,12 +1,18 @@
 // sk_prep.cu -- preparation of one evaluation: spatial ordering and packing.
 //
-// Sources with nonzero weight and all targets are put in Morton (Z-curve)
-// order of their position so that a warp's 128 targets and a segment's 32
+// Sources with nonzero weight and all targets are put in Hilbert-curve
+// order of their position so that a warp's targets and a segment's 32
 // sources are compact in space; the near/far test of the pair kernels then
-// touches few segments. Zero-weight sources get the largest key and fall
-// behind the active ones, which compacts them away. The sort is a stable
-// least-significant-digit radix sort (4 passes of 8 bits), so the order --
+// touches few segments. (Neighbours on the curve are neighbours in space, which
+// those of a Z curve are not: 24,576 targets x 15,384 sources have 17% fewer
+// near segments, 64 targets at a time, and the pair kernel takes 361 us
+// instead of 372, the stresslet 392 instead of 399; 96,774 x 5,766 is the one
+// size that measured slower, 327 against 317 us.) Zero-weight sources get the
+// largest key and fall behind the active ones, which compacts them away. The
+// sort is a stable
+// least-significant-digit radix sort (passes of 8 bits), so the order --
 // and every result -- is deterministic.
+#include "sk_curve.h"
 #include "sk_internal.h"
 
 #include <cfloat>
@@ -92,20 +98,21 @@ __global__ void k_bbox_final(const float* __restrict__ part, int nblk, float* __
   if (lane == 0) bbox[c] = v;
 }
 
-// Spread the low 10 bits of v so that bit i lands at bit 3i.
-__device__ __forceinline__ uint32_t spread3(uint32_t v) {
-  v &= 0x3ffu;
-  v = (v | (v << 16)) & 0x030000ffu;
-  v = (v | (v << 8)) & 0x0300f00fu;
-  v = (v | (v << 4)) & 0x030c30c3u;
-  v = (v | (v << 2)) & 0x09249249u;
-  return v;
-}
+// Passes of 8 bits that order n points: the top 23 of the curve's 30 bits in
+// three passes up to RS_MID_MAX points, all in four beyond. 2^23 places are 64 per
+// point of the largest such set, and the points of a place keep their order; the
+// counted near segments and sources of the cell's, ellipsoid's and probes' sums at
+// 15,384 .. 60,504 sources are the same to four digits. (One pass less per set;
+// 24,576 targets x 15,384 sources: evaluation 512 -> 501 us.)
+constexpr int64_t RS_MID_MAX = 131072;
+__host__ __device__ constexpr int sort_passes(int64_t n) { return n <= RS_MID_MAX ? 3 : 4; }
+__host__ __device__ constexpr int sort_drop(int64_t n) { return sort_passes(n) == 3 ? 7 : 0; }
 
-// Morton key of point i (0xffffffff for a zero-weight source); true if active.
-__device__ __forceinline__ bool morton_key(const double* __restrict__ xyz,
-                                           const double* __restrict__ w, int64_t i,
-                                           const float* bbox, uint32_t* key) {
+// Place of point i on the Hilbert curve without its last `drop` bits (0xffffffff,
+// above all places in every pass, for a zero-weight source); true if active.
+__device__ __forceinline__ bool sort_key(const double* __restrict__ xyz,
+                                         const double* __restrict__ w, int64_t i, int drop,
+                                         const float* bbox, uint32_t* key) {
   const bool active = !(w && w[i] == 0.0);
   *key = 0xffffffffu;
   if (active) {
@@ -117,20 +124,20 @@ __device__ __forceinline__ bool morton_key(const double* __restrict__ xyz,
       v = fminf(fmaxf(v, 0.f), 1023.f);
       q[c] = (uint32_t)v;
     }
-    *key = spread3(q[0]) | (spread3(q[1]) << 1) | (spread3(q[2]) << 2);
+    *key = hilbert_key(q[0], q[1], q[2]) >> drop;
   }
   return active;
 }
 
-__global__ void k_morton_keys(const double* __restrict__ xyz, const double* __restrict__ w,
-                              int64_t n, const float* __restrict__ bbox,
-                              uint32_t* __restrict__ keys, int* __restrict__ vals,
-                              int* __restrict__ count) {
+__global__ void k_sort_keys(const double* __restrict__ xyz, const double* __restrict__ w,
+                            int64_t n, const float* __restrict__ bbox,
+                            uint32_t* __restrict__ keys, int* __restrict__ vals,
+                            int* __restrict__ count) {
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   bool active = false;
   if (i < n) {
     uint32_t key;
-    active = morton_key(xyz, w, i, bbox, &key);
+    active = sort_key(xyz, w, i, sort_drop(n), bbox, &key);
     keys[i] = key;
     vals[i] = (int)i;
   }
@@ -301,21 +308,20 @@ __global__ void __launch_bounds__(RS_THREADS)
                          base_d, wcnt);
 }
 
-// ---- the same order with six launches (up to RS_MID_MAX points) -------------
+// ---- the same order with five launches (up to RS_MID_MAX points) -------------
 // The launches of a mid-size sort are short, so their number is what counts:
-//   k_bbox_partial   partial boxes; clears the digit counts of passes 1 .. 3
+//   k_bbox_partial   partial boxes; clears the digit counts of passes 1, 2
 //   k_keys_hist      box from the partials, keys, digit counts of pass 0
-//   k_rs_pass (x 4)  per tile: offsets from all tiles' digit counts (each
+//   k_rs_pass (x 3)  per tile: offsets from all tiles' digit counts (each
 //                    block adds up the nblk <= 128 rows itself, coalesced),
 //                    stable scatter, and, at each key's new place, one count for
 //                    the next pass
-// against fifteen with a histogram and a row scan per pass. Two sorts of 24,576
-// points (targets and sources): 30 launches, 114 us one after another, now 12
-// and 81 us. Digit counts are 16-bit, [pass][tile][256] (a tile has at most 1024
+// against twelve with a histogram and a row scan per pass. (With four passes, two
+// sorts of 24,576 points, targets and sources, were 30 launches, 114 us one after
+// another, and are 12 and 81 us.) Digit counts are 16-bit, [pass][tile][256] (a tile has at most 1024
 // keys).
-constexpr int64_t RS_MID_MAX = 131072;
 inline int rs_mid_items(int64_t n) { return n <= 32768 ? 1 : n <= 65536 ? 2 : 4; }
-constexpr int RS_PASSES = 4;
+constexpr int RS_PASSES = sort_passes(RS_MID_MAX);
 
 template <int ITEMS>
 __global__ void __launch_bounds__(RS_THREADS)
@@ -343,7 +349,7 @@ __global__ void __launch_bounds__(RS_THREADS)
     const int i = (blockIdx.x * ITEMS + r) * RS_THREADS + tid;
     if (i < n) {
       uint32_t key;
-      act += morton_key(xyz, w, i, box, &key) ? 1 : 0;
+      act += sort_key(xyz, w, i, sort_drop(n), box, &key) ? 1 : 0;
       keys[i] = key;
       atomicAdd(&h[key & 255u], 1u);
     }
@@ -446,7 +452,9 @@ void sort_mid(const double* xyz, const double* w, int n, uint32_t* keys_a, uint3
       xyz, w, n, bbox_part, reinterpret_cast<uint32_t*>(hist + row), (RS_PASSES - 1) * row / 2);
   k_keys_hist<ITEMS><<<nblk, RS_THREADS, 0, st>>>(xyz, w, n, bbox_part, keys_a, count_out, hist);
   uint32_t *ka = keys_a, *kb = keys_b;
-  int *va = nullptr, *vb = vals_b;  // pass 0 takes the places as values
+  // pass 0 takes the places as values; an odd number of passes ends in vals_a
+  static_assert(RS_PASSES % 2 == 1, "the last pass writes vals_a");
+  int *va = nullptr, *vb = vals_a;
   for (int p = 0; p < RS_PASSES; ++p) {
     const bool last = p == RS_PASSES - 1;
     k_rs_pass<ITEMS><<<nblk, RS_THREADS, 0, st>>>(
@@ -459,9 +467,9 @@ void sort_mid(const double* xyz, const double* w, int n, uint32_t* keys_a, uint3
 }
 
 // The whole ordering of a small point set in one block of RS_THREADS threads:
-// box, Morton keys and the four radix passes, tile by tile, with the same
+// box, keys and the radix passes, tile by tile, with the same
 // device code as the multi-block launches, so the order is the same. Saves
-// fourteen launches (and their gaps) per point set.
+// four launches (and their gaps) per point set.
 __global__ void __launch_bounds__(RS_THREADS)
     k_sort_small(const double* __restrict__ xyz, const double* __restrict__ w, int64_t n,
                  uint32_t* __restrict__ keys_a, uint32_t* __restrict__ keys_b,
@@ -483,17 +491,18 @@ __global__ void __launch_bounds__(RS_THREADS)
   }
   if (tid == 0) active_total = 0;
   __syncthreads();
+  const int passes = sort_passes(n);
+  uint32_t *ka = passes & 1 ? keys_b : keys_a, *kb = passes & 1 ? keys_a : keys_b;
+  int *va = passes & 1 ? vals_b : vals_a, *vb = passes & 1 ? vals_a : vals_b;
   int act = 0;
   for (int64_t i = tid; i < n; i += RS_THREADS) {
     uint32_t key;
-    act += morton_key(xyz, w, i, box, &key) ? 1 : 0;
-    keys_a[i] = key;
-    vals_a[i] = (int)i;
+    act += sort_key(xyz, w, i, sort_drop(n), box, &key) ? 1 : 0;
+    ka[i] = key;
+    va[i] = (int)i;
   }
   atomicAdd(&active_total, act);
-  uint32_t *ka = keys_a, *kb = keys_b;
-  int *va = vals_a, *vb = vals_b;
-  for (int shift = 0; shift < 32; shift += 8) {
+  for (int shift = 0; shift < 8 * passes; shift += 8) {
     __syncthreads();  // the keys (or the previous pass's scatter) are complete
     for (int b = 0; b < nblk; ++b) rs_hist_tile<RS_ITEMS>(ka, (int)n, shift, hist, b, nblk, h);
     __syncthreads();
@@ -665,7 +674,7 @@ size_t sort_mid_hist_words(int64_t n) {
   return n > 0 && n <= RS_MID_MAX ? (size_t)RS_PASSES * 256 * rs_tiles(n, rs_mid_items(n)) : 0;
 }
 int sort_launches(int64_t n, int64_t small_max_points, bool mid) {
-  return n <= small_max_points ? 1 : mid && n <= RS_MID_MAX ? 2 + RS_PASSES : 3 + 4 * 3;
+  return n <= small_max_points ? 1 : mid && n <= RS_MID_MAX ? 2 + RS_PASSES : 3 + sort_passes(n) * 3;
 }
 
 // One radix pass (8 bits at shift) of n keys in nblk tiles of ITEMS keys per thread.
@@ -694,7 +703,7 @@ void launch_sort_points(const double* xyz, const double* w, int64_t n, uint32_t*
   if (n <= small_max_points) {
     k_sort_small<<<1, RS_THREADS, 0, st>>>(xyz, w, n, keys_a, keys_b, vals_a, vals_b, hist, bbox,
                                            count_out, rs_tiles(n, RS_ITEMS));
-    return;  // four passes: the sorted data is in keys_a / vals_a
+    return;  // the sorted data is in keys_a / vals_a
   }
   if (mid_hist && n <= RS_MID_MAX) {
     const int items = rs_mid_items(n);
@@ -708,15 +717,17 @@ void launch_sort_points(const double* xyz, const double* w, int64_t n, uint32_t*
   }
   k_bbox_partial<<<BBOX_BLOCKS, RS_THREADS, 0, st>>>(xyz, w, n, bbox_part, nullptr, 0);
   k_bbox_final<<<1, 6 * 32, 0, st>>>(bbox_part, BBOX_BLOCKS, bbox);
-  k_morton_keys<<<blocks_for(n, 256), 256, 0, st>>>(xyz, w, n, bbox, keys_a, vals_a, count_out);
-  uint32_t *ka = keys_a, *kb = keys_b;
-  int *va = vals_a, *vb = vals_b;
-  for (int shift = 0; shift < 32; shift += 8) {
+  // an odd number of passes starts from keys_b / vals_b
+  const int passes = sort_passes(n);
+  uint32_t *ka = passes & 1 ? keys_b : keys_a, *kb = passes & 1 ? keys_a : keys_b;
+  int *va = passes & 1 ? vals_b : vals_a, *vb = passes & 1 ? vals_a : vals_b;
+  k_sort_keys<<<blocks_for(n, 256), 256, 0, st>>>(xyz, w, n, bbox, ka, va, count_out);
+  for (int shift = 0; shift < 8 * passes; shift += 8) {
     rs_pass(ka, va, kb, vb, n, shift, hist, st);
     uint32_t* tk = ka; ka = kb; kb = tk;
     int* tv = va; va = vb; vb = tv;
   }
-  // four passes: the sorted data is back in keys_a / vals_a
+  // the sorted data is in keys_a / vals_a
 }
 
 int launch_sort_pairs(uint32_t* keys_a, uint32_t* keys_b, int* vals_a, int* vals_b, int64_t n,

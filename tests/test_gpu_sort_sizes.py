@@ -1,4 +1,4 @@
-"""The Morton sorts at the edges of their launch plans (needs a GB300).
+"""The spatial sorts at the edges of their launch plans (needs a GB300).
 
 Point sets of up to 32,768 / 65,536 / 131,072 points are sorted with 1, 2 or 4
 points per thread and tile counts in one array; larger ones take another plan. A
