@@ -1269,7 +1269,7 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
       cudaMemcpyAsync(cv.plan, h_plan.data(), h_plan.size() * sizeof(int),
                       cudaMemcpyHostToDevice, st);
       int meta[N_META] = {};
-      meta[META_NS] = (int)near_slots;  // the overflow rescan's range
+      meta[META_NS_PAD] = (int)near_slots;  // the overflow rescan's range
       cudaMemcpyAsync(cv.meta, meta, sizeof(meta), cudaMemcpyHostToDevice, st);
       cudaMemsetAsync(cv.flags, 0, N_FLAGS * sizeof(unsigned long long), st);
       cudaMemsetAsync(cv.near_cnt, 0, (m_slots / NEAR_GROUP_MIN) * sizeof(int), st);

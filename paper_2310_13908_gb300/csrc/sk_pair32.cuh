@@ -1098,7 +1098,7 @@ __device__ __forceinline__ void rescan_target(const OverflowArgs& a, int64_t t, 
   const float hx = (float)x.x, hy = (float)x.y, hz = (float)x.z;
   const float lx = (float)(x.x - (double)hx), ly = (float)(x.y - (double)hy),
               lz = (float)(x.z - (double)hz);
-  const int Ns = a.meta[META_NS];
+  const int Ns = a.meta[META_NS_PAD];  // padding lies at PAD_POS, with src_orig -1
   u0 = u1 = u2 = 0;
   for (int s = lane; s < Ns; s += 32) {
     const float4 blo = a.segbox[2 * (s / SEG)], bhi = a.segbox[2 * (s / SEG) + 1];
@@ -1108,7 +1108,8 @@ __device__ __forceinline__ void rescan_target(const OverflowArgs& a, int64_t t, 
     const float4 p0 = a.srcF[(size_t)s * V], p1 = a.srcF[(size_t)s * V + 1];
     const float dx = __fadd_rn(tx, p0.x), dy = __fadd_rn(ty, p0.z), dz = __fadd_rn(tz, p1.x);
     const float r2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
-    if (r2 < rt2) Near64<L>::eval(x, a.xyz, a.w, a.dens, a.nrm, a.src_orig[s], a.scale, invd, u0, u1, u2);
+    const int j = a.src_orig[s];
+    if (r2 < rt2 && j >= 0) Near64<L>::eval(x, a.xyz, a.w, a.dens, a.nrm, j, a.scale, invd, u0, u1, u2);
   }
   for (int o = 16; o > 0; o >>= 1) {
     u0 += __shfl_xor_sync(FULL, u0, o);
