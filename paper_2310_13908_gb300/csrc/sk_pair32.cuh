@@ -37,6 +37,7 @@
 
 #include "sk_internal.h"
 #include "sk_erfc_scaled.h"
+#include "sk_near_box.h"
 #include "sk_series.cuh"
 
 // unroll factor of the far loop over the 32 sources of a segment
@@ -154,14 +155,6 @@ __device__ __forceinline__ float2 shift_residual2(float2 hi, float2 lo, float c,
   const float2 nc = make_float2(-c, -c);
   const float2 a = add2(hi, nc);  // fl(hi - c), the first rounding of shift_to_segment2
   return add2(two_sum_err2(hi, nc, a), two_sum_err2(a, lo, t));
-}
-
-// Margin added to rho_c delta in the segment-versus-warp box test: the boxes
-// hold absolute FP32 coordinates, while pair distances come from frame-
-// relative coordinates; the two differ by a few FP32 roundings of the
-// coordinates' magnitude.
-__device__ __forceinline__ float box_margin(float coord_max, float rc) {
-  return 1.0e-6f * (coord_max + rc);
 }
 
 // Near pairs (rho < rho_T) are listed per target group: the 64 * NP targets
@@ -422,37 +415,25 @@ struct LaneTgt {
   Tgt2 t[NP];
 };
 
-// The box of a warp's targets and the squared distance (with margins) within
-// which a source may have a pair inside rho_c delta with one of them: seven
-// numbers, kept one per lane in the warp's target columns (component z of slot
-// 4 of the first target pair), so that they take no registers in the far loop.
-struct WarpBox {
-  float lo[3], hi[3], r2;
-  // ts: the calling thread's column
-  template <int TPB>
-  __device__ __forceinline__ static WarpBox load(const float4* ts) {
-    const float* b = reinterpret_cast<const float*>(ts - (threadIdx.x & 31) + 4 * TPB) + 2;
-    return {{b[0], b[4], b[8]}, {b[12], b[16], b[20]}, b[24]};
-  }
-  // squared distance from the box to [l, h] (per axis), at most r2?
-  __device__ __forceinline__ bool reaches(float3 l, float3 h) const {
-    const float dx = fmaxf(0.f, fmaxf(l.x - hi[0], lo[0] - h.x));
-    const float dy = fmaxf(0.f, fmaxf(l.y - hi[1], lo[1] - h.y));
-    const float dz = fmaxf(0.f, fmaxf(l.z - hi[2], lo[2] - h.z));
-    return dx * dx + dy * dy + dz * dz < r2;
-  }
-};
+// The warp's NearBox: seven numbers, kept one per lane in the warp's target columns
+// (component z of slot 4 of the first target pair), so that they take no registers
+// in the far loop. ts: the calling thread's column.
+template <int TPB>
+__device__ __forceinline__ NearBox load_box(const float4* ts) {
+  const float* b = reinterpret_cast<const float*>(ts - (threadIdx.x & 31) + 4 * TPB) + 2;
+  return {{b[0], b[4], b[8]}, {b[12], b[16], b[20]}, b[24]};
+}
 
 // Sources of a segment that may have such a pair: lane j tests source j
 // against the box, one step for the 32 sources. (sx, sy, sz): the segment's
 // frame, to which the record's position is relative.
 template <int V>
-__device__ __forceinline__ unsigned sources_near_box(const WarpBox& wb, const float4* SS, float sx,
+__device__ __forceinline__ unsigned sources_near_box(const NearBox& wb, const float4* SS, float sx,
                                                      float sy, float sz) {
   const float4* r = SS + (threadIdx.x & 31) * V;
   const float4 a = r[0];  // {-x, -x, -y, -y}
-  const float3 x = make_float3(sx - a.x, sy - a.z, sz - r[1].x);
-  return __ballot_sync(FULL, wb.reaches(x, x));
+  return __ballot_sync(FULL, wb.reaches(source_span(sx, a.x), source_span(sy, a.z),
+                                        source_span(sz, r[1].x)));
 }
 
 // Four consecutive sources of a segment by the far formula.
@@ -492,7 +473,7 @@ __device__ __noinline__ LaneAcc<NP> general_segment(LaneAcc<NP> acc, LaneTgt<NP>
                                                     unsigned* near_idx,
                                                     unsigned long long* flags) {
   constexpr int V = L::V;
-  const unsigned near_src = sources_near_box<V>(WarpBox::load<TPB>(ts), SS, sx, sy, sz);
+  const unsigned near_src = sources_near_box<V>(load_box<TPB>(ts), SS, sx, sy, sz);
 #pragma unroll
   for (int p = 0; p < NP; ++p) tg.t[p].template load_radii<TPB>(ts + p * TGT_SLOTS * TPB);
   NearMask<NP> nm{};
@@ -563,7 +544,7 @@ __device__ __noinline__ LaneAcc<NP> exact_segment(
     const float4* __restrict__ ylo, const int* orig, const float4* ts, float sx, float sy, float sz, float hs, int64_t group,
     int* near_cnt, unsigned* near_idx, unsigned long long* flags) {
   constexpr int V = L::V;
-  const unsigned near_src = sources_near_box<V>(WarpBox::load<TPB>(ts), SS, sx, sy, sz);
+  const unsigned near_src = sources_near_box<V>(load_box<TPB>(ts), SS, sx, sy, sz);
   NearMask<NP> nm{};
 #pragma unroll 1
   for (int j = 0; j < SEG; ++j) {
@@ -783,7 +764,7 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
                              fmaxf(fabsf(blo[2]), fabsf(bhi[2])));
     const float rm = rc * 1.00005f + box_margin(cmax, rc);
     rc2test = rm * rm;
-    // the warp's box, one component per lane (WarpBox)
+    // the warp's box, one component per lane (load_box)
     const float v = lane < 3 ? (lane == 0 ? blo[0] : lane == 1 ? blo[1] : blo[2])
                     : lane < 6 ? (lane == 3 ? bhi[0] : lane == 4 ? bhi[1] : bhi[2]) : rc2test;
     reinterpret_cast<float*>(ts + 4 * TPB)[2] = v;
@@ -864,9 +845,10 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
         // its registers (cell of 24,576 nodes 415 -> 401 us, 96,774 sources x
         // 5,766 targets 494 -> 449 us); two pairs: from registers (the
         // stresslet at 221,184 nodes 20.3 -> 19.8 ms)
-        WarpBox wb{{blo[0], blo[1], blo[2]}, {bhi[0], bhi[1], bhi[2]}, rc2test};
-        if constexpr (NP == 1) wb = WarpBox::load<TPB>(ts);
-        nb = wb.reaches(make_float3(lo.x, lo.y, lo.z), make_float3(hi.x, hi.y, hi.z));
+        NearBox wb{{blo[0], blo[1], blo[2]}, {bhi[0], bhi[1], bhi[2]}, rc2test};
+        if constexpr (NP == 1) wb = load_box<TPB>(ts);
+        nb = wb.reaches(segment_span(lo.x, hi.x), segment_span(lo.y, hi.y),
+                        segment_span(lo.z, hi.z));
         csx = frame_mid(lo.x, hi.x);
         csy = frame_mid(lo.y, hi.y);
         csz = frame_mid(lo.z, hi.z);
