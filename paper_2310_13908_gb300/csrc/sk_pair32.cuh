@@ -787,6 +787,10 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
 
   // ---- source pipeline: no CTA-wide barrier inside the loop; the last warp
   // to release a stage issues the next bulk copy into it.
+  // The server's CTAs run item after item: the previous item's loads from the stages
+  // and its finish's stores there are ordered before the bulk copies below, which
+  // write through the async proxy.
+  if constexpr (kFresh) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();  // the previous item (if any) no longer uses the stages
   if (tid == 0) {
     for (int b = 0; b < STAGES; ++b) {
