@@ -784,7 +784,7 @@ __global__ void k_fmm_pack_near(const double* __restrict__ X, const double* __re
     g1 = (float)(ws * f[3 * i + 1]);
     g2 = (float)(ws * f[3 * i + 2]);
   }
-  write_sl_record(srcF + s * V_SL, x, y, z, g0, g1, g2);
+  write_sl_record(srcF + s * V_SL, x, y, z, g0, g1, g2, real);
   src_orig[s] = (int)i;
 }
 
@@ -797,26 +797,31 @@ __global__ void k_fmm_pack_eq(const double* __restrict__ box, const double* __re
   const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (s >= (int64_t)k * eqp) return;  // k * eqp is a multiple of SEG
   const int j = (int)(s / eqp), q = (int)(s % eqp);
-  const bool real = q < Np && count[j] > 0;
+  const bool used = count[j] > 0, real = used && q < Np;
+  // padding repeats the cluster's last point, without density: like the others it
+  // is out of every target's near range, and src_orig has no entry for it
   double ex = PAD_POS, ey = PAD_POS, ez = PAD_POS;
-  if (real) {
+  if (used) {
     const double a = box[4 * j + 3];
-    ex = box[4 * j] + R_EQUIV * a * unit[3 * q];
-    ey = box[4 * j + 1] + R_EQUIV * a * unit[3 * q + 1];
-    ez = box[4 * j + 2] + R_EQUIV * a * unit[3 * q + 2];
+    const double* u = unit + 3 * min(q, Np - 1);
+    ex = box[4 * j] + R_EQUIV * a * u[0];
+    ey = box[4 * j + 1] + R_EQUIV * a * u[1];
+    ez = box[4 * j + 2] + R_EQUIV * a * u[2];
   }
   const float3 c = warp_box(real, (float)ex, (float)ey, (float)ez, segbox + 2 * ((base + s) / SEG));
   float x = PAD_POS, y = PAD_POS, z = PAD_POS, g0 = 0.f, g1 = 0.f, g2 = 0.f;
-  if (real) {
+  if (used) {
     x = (float)(ex - (double)c.x);
     y = (float)(ey - (double)c.y);
     z = (float)(ez - (double)c.z);
+  }
+  if (real) {
     const double* ph = phi + ((int64_t)j * Np + q) * 3;
     g0 = (float)(ph[0] * scale);
     g1 = (float)(ph[1] * scale);
     g2 = (float)(ph[2] * scale);
   }
-  write_sl_record(srcF + (base + s) * V_SL, x, y, z, g0, g1, g2);
+  write_sl_record(srcF + (base + s) * V_SL, x, y, z, g0, g1, g2, used);
 }
 
 // Targets box by box (each box's targets in curve order, padded to whole

@@ -104,9 +104,10 @@ __device__ __forceinline__ float3 warp_box(bool real, float x, float y, float z,
 
 // Single-layer FP32 source record (duplicated lanes for f32x2 arithmetic):
 // {-x,-x,-y,-y} {-z,-z,gx,gx} {gy,gy,gz,gz}, x relative to the segment frame.
+// Padding (!real) has two different x, which marks it (sources_near_box).
 __device__ __forceinline__ void write_sl_record(float4* o, float x, float y, float z, float g0,
-                                                float g1, float g2) {
-  o[0] = make_float4(-x, -x, -y, -y);
+                                                float g1, float g2, bool real) {
+  o[0] = make_float4(-x, real ? -x : -2.f * x, -y, -y);
   o[1] = make_float4(-z, -z, g0, g0);
   o[2] = make_float4(g1, g1, g2, g2);
 }

@@ -426,14 +426,15 @@ __device__ __forceinline__ NearBox load_box(const float4* ts) {
 
 // Sources of a segment that may have such a pair: lane j tests source j
 // against the box, one step for the 32 sources. (sx, sy, sz): the segment's
-// frame, to which the record's position is relative.
+// frame, to which the record's position is relative. Never padding (write_sl_record):
+// at a delta of 1e15 and more it lies near targets, and a near list must not name it.
 template <int V>
 __device__ __forceinline__ unsigned sources_near_box(const NearBox& wb, const float4* SS, float sx,
                                                      float sy, float sz) {
   const float4* r = SS + (threadIdx.x & 31) * V;
   const float4 a = r[0];  // {-x, -x, -y, -y}
-  return __ballot_sync(FULL, wb.reaches(source_span(sx, a.x), source_span(sy, a.z),
-                                        source_span(sz, r[1].x)));
+  return __ballot_sync(FULL, a.x == a.y && wb.reaches(source_span(sx, a.x), source_span(sy, a.z),
+                                                      source_span(sz, r[1].x)));
 }
 
 // Four consecutive sources of a segment by the far formula.
@@ -526,6 +527,8 @@ __device__ __noinline__ LaneAcc<NP> general_segment(LaneAcc<NP> acc, LaneTgt<NP>
       }
     }
   }
+#pragma unroll
+  for (int b = 0; b < 2 * NP; ++b) nm.m[b] &= near_src;  // no padding beside a source in reach
   near_append_warp<NP, kFresh>(nm, group, orig, near_cnt, near_idx, flags);
   return acc;
 }
@@ -579,6 +582,8 @@ __device__ __noinline__ LaneAcc<NP> exact_segment(
       for (int p = 0; p < NP; ++p) L::far(src, dx[p], dy[p], dz[p], r2[p], acc.u[p]);
     }
   }
+#pragma unroll
+  for (int b = 0; b < 2 * NP; ++b) nm.m[b] &= near_src;  // no padding beside a source in reach
   near_append_warp<NP, kFresh>(nm, group, orig, near_cnt, near_idx, flags);
   return acc;
 }

@@ -578,7 +578,7 @@ __global__ void k_pack_src32(const double* __restrict__ xyz, const double* __res
     }
   }
   float4* o = srcF + s * V;
-  write_sl_record(o, x, y, z, d0, d1, d2);
+  write_sl_record(o, x, y, z, d0, d1, d2, real);
   if (LAYER == LAYER_DL) {
     o[3] = make_float4(n0, n0, n1, n1);
     o[4] = make_float4(n2, n2, 0.f, 0.f);
