@@ -137,16 +137,23 @@ __device__ __forceinline__ float near_radius2(float rc2, float ratio) {
 
 // 1/sqrt(x): the hardware's approximation y0 (about 20 bits, one instruction)
 // and one step of Householder's cubic iteration, y0 (1 + e/2 + 3/8 e^2) with
-// e = 1 - x y0^2; the term left out is below 2^-60. Overflowed x gives 0.
+// e = 1 - x y0^2; the term left out, 5/16 e^3, is below 2^-58. With the roundings of
+// y0^2 and of the last step the result is within 2^-53 + 2^-54 + 2^-58 of 1/sqrt(x).
+// The approximation flushes subnormal x: they, 0, infinity, NaN and negative x go to
+// the library function.
 __device__ __forceinline__ double rsqrt_fp64(double x) {
+  if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7fe00000u) return rsqrt(x);
   double y0;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
-  const double e = __double2hiint(x) < 0x7ff00000 ? fma(-x, y0 * y0, 1.0) : 0.0;
+  const double e = fma(-x, y0 * y0, 1.0);
   return fma(y0, e * fma(0.375, e, 0.5), y0);
 }
 
-// 1/x the same way (reciprocal approximation and one cubic step).
+// 1/x the same way: the approximation y0 and a cubic step of Newton's series for the
+// reciprocal, y0 (1 + e + e^2), e = 1 - x y0; within 2^-53 + 2^-58. For
+// 2^-1022 <= x < 2^1021 (1/x is normal too); any other x is divided.
 __device__ __forceinline__ double rcp_fp64(double x) {
+  if ((unsigned)__double2hiint(x) - 0x00100000u >= 0x7fc00000u) return 1.0 / x;
   double y0;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
   const double e = fma(-x, y0, 1.0);

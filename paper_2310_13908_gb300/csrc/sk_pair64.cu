@@ -215,6 +215,11 @@ __global__ void __launch_bounds__(TPB64, 2)
     bhi[c] += pad;
   }
   const float rc2test = rc2max * 1.0001f;
+  // Warps with a target whose 1/delta^2 overflows (delta below 7.5e-155) decide pair by
+  // pair: there y does not tell r > 0 from far (a smoothed pair's 1/delta^3 would
+  // overflow, so only r = 0 takes the table).
+  const bool pair_by_pair = __any_sync(FULL, invd2[0] == DBL_MAX || invd2[1] == DBL_MAX);
+  const unsigned table_hi = pair_by_pair ? 0u : Y_TABLE_HI;
 
   double u[2][3] = {{0, 0, 0}, {0, 0, 0}};  // far pairs
   double v[2][3] = {{0, 0, 0}, {0, 0, 0}};  // near pairs, times delta
@@ -279,14 +284,16 @@ __global__ void __launch_bounds__(TPB64, 2)
             // runs one of the two forms; beyond the smoothed range both give
             // the plain kernel.
             if (__any_sync(FULL, hi[0] < Y_NEAR_HI || hi[1] < Y_NEAR_HI)) {
-              if (__all_sync(FULL, hi[0] < Y_TABLE_HI && hi[1] < Y_TABLE_HI)) {
+              if (__all_sync(FULL, hi[0] < table_hi && hi[1] < table_hi)) {
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
                   near64<LAYER>(tab, G, Nn, dx[h], dy[h], dz[h], y[h], invd2[h], v[h]);
               } else {
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                  if (hi[h] < Y_TABLE_HI)
+                  bool in_table = hi[h] < Y_TABLE_HI;
+                  if (pair_by_pair && invd2[h] == DBL_MAX) in_table = r2[h] == 0.0;
+                  if (in_table)
                     near64<LAYER>(tab, G, Nn, dx[h], dy[h], dz[h], y[h], invd2[h], v[h]);
                   else
                     far64<LAYER>(G, Nn, dx[h], dy[h], dz[h], r2[h], u[h]);
