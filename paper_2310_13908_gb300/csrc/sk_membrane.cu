@@ -227,15 +227,19 @@ constexpr int SLOPE_LINES = 8;  // grid lines per CTA
 __host__ __device__ constexpr int slope_run(int n, int L) { return (n - 2 + L - 1) / L; }
 
 // The value entering lane sub's run from the D lanes on its DIR side: run r
-// maps its entering value x to A x + B.
+// maps its entering value x to A x + B. A value that is not finite reaches its whole
+// line, as the recurrence has it, not the next D runs only.
 template <int L, int DIR>
 __device__ __forceinline__ double entering(double A, double B, int sub, int D) {
+  const unsigned bad = __ballot_sync(0xffffffffu, (__double2hiint(B) & 0x7ff00000) == 0x7ff00000);
+  const unsigned line = (L == 32 ? 0xffffffffu : (1u << L) - 1u) << ((threadIdx.x & 31) / L * L);
+  const int reach = (bad & line) ? L - 1 : D;
   double x = 0.0;
-  for (int d = D; d >= 1; --d) {
+  for (int d = bad ? L - 1 : D; d >= 1; --d) {
     const int from = sub - DIR * d;
     const double b = __shfl_sync(0xffffffffu, B, from, L);
     const double a = __shfl_sync(0xffffffffu, A, from, L);
-    if (from >= 0 && from < L) x = fma(a, x, b);
+    if (d <= reach && from >= 0 && from < L) x = fma(a, x, b);
   }
   return x;
 }
