@@ -523,7 +523,7 @@ __device__ __forceinline__ Frame frame_at(const double* __restrict__ t6, int64_t
   // one reciprocal square root for W and 1/W (a square root and divisions
   // take several times the FP64 instructions)
   const double W2 = fr.E * fr.G - fr.F * fr.F;
-  if (W2 > 1e-290) {
+  if (W2 > 1e-290 && W2 < INFINITY) {
     fr.iW = rsqrt_fp64(W2);
     fr.W = W2 * fr.iW;
   } else {
