@@ -234,6 +234,7 @@ struct Slot {
   EvalBufs b;
   int* tb_counters = nullptr;  // [n_tb + 1]
   unsigned seq = 0;
+  float rt_ratio = 0.f;  // near_radius2's ratio, of the thresholds that the preparation read
   cudaEvent_t prep_done = nullptr, copy_done = nullptr, update_done = nullptr;
   // fork and join of the target sort onto the preparation stream's partner
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
@@ -336,6 +337,18 @@ void launch_kernel(sk_server* srv, bool capsules) {
 // follow one another on its stream.
 int capsule_set(int slot) { return slot % SERVE_PREP_STREAMS; }
 
+// Preparation kernels of the slot's evaluation on st, at the context's thresholds of
+// this moment: the target records hold rho_c^2 delta^2, from which the items take
+// rho_T^2 delta^2 by the same thresholds' ratio, also if they are set anew before
+// the items are published.
+void enqueue_slot_prep(sk_server* srv, Slot& sl, int slot, cudaStream_t st) {
+  const double rho_T = srv->ctx->rho_T, rho_c = srv->ctx->rho_c;
+  sl.rt_ratio = near_ratio(rho_T, rho_c);
+  const PrepFork pf{srv->s_prep_aux[slot % SERVE_PREP_STREAMS], sl.fork_ev, sl.join_ev};
+  enqueue_prep(sl.req->shape, sl.b, rho_T, rho_c, st, &pf);
+  cudaEventRecord(sl.prep_done, st);
+}
+
 // One step of a capsule request, on st: the inputs of its sum (membrane
 // force, weights, delta* at the current nodes), cleared counters and the
 // preparation kernels; the step's items are published when st reaches
@@ -345,9 +358,7 @@ void enqueue_capsule_step(sk_server* srv, Slot& sl, int slot, cudaStream_t st) {
   capsule_enqueue_step_inputs(r->cap, sl.b, st, capsule_set(slot));
   const int n_tb = (int)(sl.b.M_pad / SERVE_TGT_CTA);
   cudaMemsetAsync(sl.tb_counters, 0, (n_tb + 1) * sizeof(int), st);
-  const PrepFork pf{srv->s_prep_aux[slot % SERVE_PREP_STREAMS], sl.fork_ev, sl.join_ev};
-  enqueue_prep(r->shape, sl.b, srv->ctx->rho_T, srv->ctx->rho_c, st, &pf);
-  cudaEventRecord(sl.prep_done, st);
+  enqueue_slot_prep(srv, sl, slot, st);
 }
 
 // Admit: bind a queued request to a free slot and its arena block, enqueue
@@ -383,9 +394,7 @@ bool admit_one(sk_server* srv, Req* r, Slot& sl, int slot) {
   cudaMemcpyAsync((void*)b.tgt_xyz, r->h_txyz, 3 * s.M * sizeof(double), cudaMemcpyHostToDevice, st);
   cudaMemcpyAsync((void*)b.delta, r->h_delta, s.n_delta * sizeof(double), cudaMemcpyHostToDevice, st);
   cudaMemsetAsync(sl.tb_counters, 0, (n_tb + 1) * sizeof(int), st);
-  const PrepFork pf{srv->s_prep_aux[slot % SERVE_PREP_STREAMS], sl.fork_ev, sl.join_ev};
-  enqueue_prep(s, b, srv->ctx->rho_T, srv->ctx->rho_c, st, &pf);
-  cudaEventRecord(sl.prep_done, st);
+  enqueue_slot_prep(srv, sl, slot, st);
   r->st.admit_us = now_us(srv);
   return true;
 }
@@ -398,8 +407,7 @@ void publish(sk_server* srv, int slot) {
   const double scale = layer_scale(s);
   SlotDesc d{};
   d.pa = PairArgs{b.srcF, b.segbox, b.src_orig, b.meta, b.tgtF, b.M_pad, b.n_chunks,
-                  b.part, b.near_cnt, b.near_idx, b.flags,
-                  near_ratio(srv->ctx->rho_T, srv->ctx->rho_c)};
+                  b.part, b.near_cnt, b.near_idx, b.flags, sl.rt_ratio};
   d.oa = OverflowArgs{b.srcF, b.segbox, b.src_orig, b.meta, b.tgtF, b.tgt64, b.near_cnt,
                       b.src_xyz, b.src_w, b.dens, b.nrm, scale, b.flags, b.near_ovf};
   d.fa = FinishArgs{b.tgt64, b.tgt_perm, b.M_pad, b.n_chunks, b.part, b.near_cnt, b.near_idx,
