@@ -157,7 +157,7 @@ double layer_scale(const EvalShape& s) {
 // sort and pack run on pf->aux beside the source sort and pack (the two touch
 // disjoint buffers; the result does not change), and `st` waits for them.
 // Returns the number of kernels launched.
-int enqueue_prep(const EvalShape& s, const EvalBufs& b, double rho_T, double rho_c,
+int enqueue_prep(const EvalShape& s, const EvalBufs& b, double rho_c,
                  cudaStream_t st, const PrepFork* pf) {
   const bool fp32 = s.precision == SK_FP32C;
   const double scale = layer_scale(s);
@@ -200,7 +200,7 @@ int enqueue_eval(const EvalShape& s, const EvalBufs& b, double rho_T, double rho
   const bool fp32 = s.precision == SK_FP32C;
   const double scale = layer_scale(s);
   if (ev) cudaEventRecord(ev[0], st);
-  int launches = enqueue_prep(s, b, rho_T, rho_c, st, pf);
+  int launches = enqueue_prep(s, b, rho_c, st, pf);
   if (ev) cudaEventRecord(ev[1], st);
   if (fp32) {
     launch_pair32(s.layer, b, rho_T, rho_c, scale, st, ev ? ev[2] : nullptr);  // with the finish

@@ -361,7 +361,7 @@ void carve_eval_buffers(Bump& bp, const EvalShape& s, EvalBufs& b);
 // choose_chunks and choose_decomposition (the split into work items): sk_decomp.h
 double layer_scale(const EvalShape& s);  // 1/(8 pi mu) or -6/(8 pi)
 // pf (optional) forks the target sort onto pf->aux when s.split_sorts.
-int enqueue_prep(const EvalShape& s, const EvalBufs& b, double rho_T, double rho_c,
+int enqueue_prep(const EvalShape& s, const EvalBufs& b, double rho_c,
                  cudaStream_t st, const PrepFork* pf = nullptr);
 // Returns the number of kernels launched. ev (optional, 4 events) brackets
 // the whole evaluation (ev[0], ev[3]) and the pair kernel (ev[1], ev[2]).

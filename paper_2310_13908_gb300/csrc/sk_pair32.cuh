@@ -1072,7 +1072,6 @@ struct FinishArgs {
   double scale;
   double* u;
   unsigned long long* flags;
-  int group = 0;  // targets per group: 64 * (f32x2 pairs per lane) of the pair kernel
 };
 
 // FP64 near sum of target t by a rescan of all packed sources with exactly the

@@ -17,7 +17,6 @@ namespace sk {
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-constexpr int SEGS64 = TILE64 / SEG;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
