@@ -54,7 +54,7 @@ extern "C" {
 /* ---- precision and memory-space selectors -------------------------------- */
 #define SK_FP64   0  /* every pair in FP64 */
 #define SK_FP32C  1  /* FP32 pairs, compensated (two-sum) accumulation per target,
-                        FP64 series for pairs with r/delta < rho_T, FP64 final sum */
+                        FP64 factors for pairs with r/delta < rho_T, FP64 final sum */
 #define SK_HOST   0  /* all array arguments are host pointers */
 #define SK_DEVICE 1  /* all array arguments are device pointers on the context's device */
 
@@ -85,8 +85,8 @@ const char* sk_last_error(const sk_ctx* ctx);
 int sk_version(void);
 
 /* Tuning knobs of the SK_FP32C path (defaults: rho_T = 0.5, rho_c = 5.0).
- *   rho_T: pairs with r/delta below it are evaluated in FP64 by power series
- *          (Sec. 3.4: s1/r and s2/r^3 are smooth at r = 0). 0 < rho_T <= 2.
+ *   rho_T: pairs with r/delta below it are evaluated in FP64, by polynomials in
+ *          r^2 (Sec. 3.4: s1/r and s2/r^3 are smooth at r = 0). 0 < rho_T <= 2.
  *   rho_c: pairs with r/delta at or above it use s1 = s2 = s3 = 1, the plain
  *          Stokeslet/stresslet. The omitted fraction of a pair's value is
  *          largest at r/delta = rho_c: at rho_c = 5 it is 1.2e-9 (s1) and
@@ -101,7 +101,7 @@ int sk_set_fp32c_thresholds(sk_ctx* ctx, double rho_T, double rho_c);
 typedef struct {
   int64_t n_src_active;      /* sources with w != 0 (the N_s of the interaction count) */
   int64_t n_tgt;             /* targets */
-  int64_t near_pairs;        /* pairs evaluated in FP64 by series (SK_FP32C) */
+  int64_t near_pairs;        /* pairs evaluated in FP64: r/delta < rho_T (SK_FP32C) */
   int64_t overflow_targets;  /* targets rescanned because their group's near-pair list
                                 overflowed (a group: the 64 or 128 targets of one warp) */
   int64_t kernel_launches;   /* CUDA kernels the evaluation launched */

@@ -155,7 +155,7 @@ def sk_last_error(ctx) -> str:
 
 
 def sk_set_fp32c_thresholds(ctx, rho_T: float, rho_c: float) -> None:
-    """SK_FP32C regime thresholds: FP64 series below rho_T, plain kernel from rho_c."""
+    """SK_FP32C regime thresholds: FP64 factors below rho_T, plain kernel from rho_c."""
     _check(ctx, load().sk_set_fp32c_thresholds(ctx, float(rho_T), float(rho_c)))
 
 

@@ -337,15 +337,15 @@ __global__ void k_km_frame(const double* __restrict__ part, int nblk, double* __
 }
 
 // One Lloyd step's assignment and the exact sums of each cluster's points:
-// every coordinate rounded to a multiple of the quantum q above the box corner (at most 2^34 quanta) and
-// added in 64-bit integers, which makes the sums independent of the order of
+// every coordinate rounded to a multiple of the quantum q above the box corner (at
+// most 2^34 quanta) and added in 64-bit integers, which makes the sums independent of the order of
 // the additions; point counts likewise. A warp first adds up the quanta of
 // its lanes that share a cluster (consecutive points mostly do), so one lane
 // per cluster and warp adds them on; for k <= KM_SMEM_SUMS a block gathers
 // those in shared memory first. (One launch: the labels of an inner step are
-// needed by nothing else, and the points are in registers. Assignment, two
-// memsets and sums took 26 + 9 us and four launches per step at 98,304 points
-// and 128 centres; now 27 us and, with the centres' update, two.)
+// needed by nothing else, and the points are in registers. 27 us at 98,304
+// points and 128 centres; as an assignment, two memsets and sums 35 us and three more
+// launches per step.)
 __global__ void __launch_bounds__(FMM_TPB) k_km_step(const double* __restrict__ X,
                                                      const double* __restrict__ w, int64_t N,
                                                      const double* __restrict__ C,

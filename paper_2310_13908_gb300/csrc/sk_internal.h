@@ -315,8 +315,8 @@ namespace sk {
 // Largest point set ordered by the single-block sort by default;
 // SK_SMALL_SORT_POINTS in the environment of sk_create overrides it per
 // context (0 turns it off). Measured (single layer, nodes as sources and
-// targets, single block / six launches, now five): 384 points 112 / 120 us, 1014 121 / 123,
-// 1176 135 / 123, 1944 145 / 127, 2904 172 / 133.
+// targets, single block / five launches): 384 points 87 / 93 us, 726 100 / 103, 1014
+// 108 / 109, 1176 110 / 100, 1944 118 / 105, 2904 136 / 109.
 constexpr int64_t SMALL_SORT_POINTS = 1024;
 
 // CTA size of the FP64 pair kernel for problems too small to fill the GPU

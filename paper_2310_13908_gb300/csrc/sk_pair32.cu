@@ -51,10 +51,10 @@ __global__ void __launch_bounds__(TPB32, MINB)
 // group of G targets, each with its share of the targets (and the whole list,
 // of which it keeps its own), the near-sum scratch in dynamic shared memory.
 // Bound by the FP64 pipe (60% busy) and the latency of its phases; small grids
-// by how many SMs get a share. Against one CTA per group with a thread per
-// target (single layer): 104 -> 72 us at 24,576 targets (64 chunks, 12 near pairs
-// per target), 47 -> 16 us at 1,944, 61 -> 22 us at 5,766; one warp per share
-// instead of four took 112 us at 24,576 targets.
+// by how many SMs get a share. Single layer: 72 us at 24,576 targets (64 chunks, 12
+// near pairs per target), 16 us at 1,944, 22 us at 5,766; one CTA per group with a
+// thread per target 104, 47 and 61 us; one warp per share instead of four 112 us at
+// 24,576 targets.
 constexpr int FIN_PARTS = 4, FIN_THREADS = 128;
 template <class L, int G>
 __global__ void __launch_bounds__(FIN_THREADS) k_finish32(OverflowArgs oa, FinishArgs a,
@@ -100,10 +100,10 @@ void launch_pair32_t(const EvalBufs& b, float rt_ratio, double scale,
   } else {
     // One pair per lane, single layer: CTAs of 128 threads. A CTA's warps meet
     // few or many segments inside rho_c delta, and the SM waits for the
-    // slowest; smaller CTAs wait less (pair kernel at 128 / 256 threads: 1,944
-    // nodes 60 / 68 us, 24,576 nodes 373 / 385 us, 96,774 sources x 5,766
-    // targets 418 / 430 us; 64 threads: slower from 24,576 nodes on). The
-    // stresslet's larger records leave room for too few of them: 417 / 405 us.
+    // slowest; smaller CTAs wait less (pair kernel with 256 threads: 1,944 nodes
+    // 13% longer, 24,576 nodes and 96,774 sources x 5,766 targets 3%; 64 threads:
+    // longer from 24,576 nodes on). The stresslet's larger records leave room for
+    // too few of them: 24,576 nodes 3% longer with 128.
     constexpr int TPB = NP == 1 && L::V == V_SL ? 128 : TPB32;
     constexpr size_t smem1 = pair_smem_bytes<L, NP, TPB>();
     const auto k = k_pair32<L, NP, TPB, MINB * (TPB32 / TPB)>;

@@ -5,11 +5,13 @@
 // Regimes per pair, rho = r/delta_x (delta of the target, Eq. regparam):
 //   rho >= rho_c          plain Stokeslet / stresslet (s_i = 1), FP32 f32x2
 //   rho_T <= rho < rho_c  closed-form s_i with erf/exp, FP32 (Sec. 3.4)
-//   rho < rho_T           recorded in a per-target list and summed in FP64
-//                         by power series (finish step), incl. r = 0
+//   rho < rho_T           listed per target group and summed in FP64 in the
+//                         finish step (local polynomials of s_i / rho^k below
+//                         rho = 0.5, sk_near_factors.h; power series and closed
+//                         forms beyond), incl. r = 0
 //
 // Work item = (block of sorted targets, chunk of source tiles). A CTA streams
-// its chunk through shared memory in tiles of 256 sources with a 3-4 stage
+// its chunk through shared memory in tiles of 256 sources with a 2 to 4 stage
 // pipeline of bulk async copies (cp.async.bulk + mbarrier); a stage is
 // released per warp, and the last warp to release it issues its next copy, so
 // no CTA-wide barrier sits in the tile loop. Per warp and per 32-source
@@ -460,11 +462,11 @@ __device__ __forceinline__ void far_four(LaneAcc<NP>& acc, const LaneTgt<NP>& tg
 // lane's pair p lies inside rho_c delta, then the regimes (which give the far
 // formula's bits for pairs beyond rho_c, so neither choice changes a result).
 // The warp appends the segment's near pairs at the end. Out of line: its
-// registers do not weigh on the far loop. On a cell of 24,576 nodes 27% of the
+// registers do not weigh on the far loop. On a cell of 24,576 nodes 24% of the
 // (warp, segment) visits come here and about half of their sources are
-// cleared; they are half of the pair kernel's time (a voted source costs about
-// four far ones). Against a vote and an append per source: pair kernel 465 ->
-// 373 us there, 139 -> 60 us at 1,944 nodes, 580 -> 418 us for 96,774 sources x
+// cleared; they are half of the pair kernel's 331 us (a voted source costs about
+// four far ones). With a vote and an append per source the pair kernel took 25%
+// longer there, 2.3 times as long at 1,944 nodes and 39% longer for 96,774 sources x
 // 5,766 targets.
 template <class L, int NP, int TPB, bool kFresh>
 __device__ __noinline__ LaneAcc<NP> general_segment(LaneAcc<NP> acc, LaneTgt<NP> tg,
@@ -486,8 +488,8 @@ __device__ __noinline__ LaneAcc<NP> general_segment(LaneAcc<NP> acc, LaneTgt<NP>
     }
     if constexpr (NP == 1 && !kFresh) {
       // two sources at a time: two independent chains per warp (the server's
-      // kernel, with three CTAs per SM, has no registers for them: 24 requests 28.5
-      // ms, with two 29.1)
+      // kernel, with three CTAs per SM, has no registers for them: a burst of
+      // 24 requests takes 27.3 ms, with two 2% longer)
 #pragma unroll 1
       for (int j = g; j < g + 4; j += 2) {
         typename L::Src src[2];
@@ -683,9 +685,9 @@ struct TileStride {
 // tiles near a target block follow one another in the sorted order; dealt out
 // to all chunks, they make its CTAs equally long, where one or two contiguous
 // chunks with all of them ran several times as long as the rest and
-// idled the chip at the end of the launch. (Pair kernel, contiguous chunks / dealt
-// out: 96,774 sources x 5,766 targets 412 / 327 us; 135,168 x 221,184, stresslet,
-// 20.73 / 19.87 ms; 239,880 x 493,216 68.84 / 67.93 ms.)
+// idled the chip at the end of the launch. (Pair kernel with contiguous
+// chunks: 96,774 sources x 5,766 targets 26% longer; 135,168 x 221,184, stresslet, 4%;
+// 239,880 x 493,216 1.3%.)
 template <bool kFresh = false>
 __device__ __forceinline__ TileStride chunk_tiles(const PairArgs& a, int ch) {
   const int n_tiles = (kFresh ? __ldcg(a.meta + META_NS_PAD) : a.meta[META_NS_PAD]) / TILE;
@@ -851,9 +853,9 @@ __device__ __forceinline__ bool pair_item(const PairArgs& a, int tb, const TL& t
         const float4 hi =
             kFresh ? __ldcg(segbox + 2 * (sg + lane) + 1) : segbox[2 * (sg + lane) + 1];
         // one pair per lane: the box from shared memory leaves the far loop
-        // its registers (cell of 24,576 nodes 415 -> 401 us, 96,774 sources x
-        // 5,766 targets 494 -> 449 us); two pairs: from registers (the
-        // stresslet at 221,184 nodes 20.3 -> 19.8 ms)
+        // its registers (otherwise 3% longer on a cell of 24,576 nodes, 10% for
+        // 96,774 sources x 5,766 targets); two pairs: from registers (otherwise
+        // 2.5% longer for the stresslet at 221,184 nodes)
         NearBox wb{{blo[0], blo[1], blo[2]}, {bhi[0], bhi[1], bhi[2]}, rc2test};
         if constexpr (NP == 1) wb = load_box<TPB>(ts);
         nb = wb.reaches(segment_span(lo.x, hi.x), segment_span(lo.y, hi.y),
@@ -1186,8 +1188,8 @@ __device__ __forceinline__ double fin_sum(double v) {
 }
 
 // v[0 .. n) (distinct), n <= 32 Q, in ascending order by one warp, each lane
-// ranking Q values (239,880 x 493,216 at delta = 3h, 36 near pairs per node: 74.0 ms
-// with runs above 32 sorted by one lane, now 70.5). Out of line: only delta >= 3h has
+// ranking Q values (239,880 x 493,216 at delta = 3h, 36 near pairs per node: 70.5 ms,
+// with runs above 32 sorted by one lane 74.0). Out of line: only delta >= 3h has
 // such runs, and what is inlined here moves the far loop's schedule.
 template <int Q>
 __device__ __noinline__ void rank_entries(unsigned* v, int n) {

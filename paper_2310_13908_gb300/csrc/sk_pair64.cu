@@ -2,7 +2,7 @@
 //
 // Same work decomposition as the FP32 kernels (sorted targets, chunks of
 // source tiles staged by bulk async copies, per-segment near/far test), all
-// arithmetic in FP64:
+// arithmetic in FP64 but the tails of the table's polynomials (terms below 2^-30):
 //   rho >= 7   plain Stokeslet / stresslet (s_i = 1 to double precision)
 //   rho < 7    s_i / rho^k from a table of local polynomials in rho^2
 //              (sk_factors64.h), incl. r = 0

@@ -5,13 +5,11 @@
 // sources are compact in space; the near/far test of the pair kernels then
 // touches few segments. (Neighbours on the curve are neighbours in space, which
 // those of a Z curve are not: 24,576 targets x 15,384 sources have 17% fewer
-// near segments, 64 targets at a time, and the pair kernel takes 361 us
-// instead of 372, the stresslet 392 instead of 399; 96,774 x 5,766 is the one
-// size that measured slower, 327 against 317 us.) Zero-weight sources get the
-// largest key and fall behind the active ones, which compacts them away. The
-// sort is a stable
-// least-significant-digit radix sort (passes of 8 bits), so the order --
-// and every result -- is deterministic.
+// near segments, 64 targets at a time, and the pair kernel takes 3% less, the
+// stresslet's 2%; 96,774 x 5,766 is the one size that measured slower, by 3%.)
+// Zero-weight sources get the largest key and fall behind the active ones, which
+// compacts them away. The sort is a stable least-significant-digit radix sort
+// (passes of 8 bits), so the order -- and every result -- is deterministic.
 #include "sk_curve.h"
 #include "sk_internal.h"
 
@@ -102,8 +100,8 @@ __global__ void k_bbox_final(const float* __restrict__ part, int nblk, float* __
 // three passes up to RS_MID_MAX points, all in four beyond. 2^23 places are 64 per
 // point of the largest such set, and the points of a place keep their order; the
 // counted near segments and sources of the cell's, ellipsoid's and probes' sums at
-// 15,384 .. 60,504 sources are the same to four digits. (One pass less per set;
-// 24,576 targets x 15,384 sources: evaluation 512 -> 501 us.)
+// 15,384 .. 60,504 sources are the same to four digits. (A fourth pass adds
+// 2% to the evaluation of 24,576 targets x 15,384 sources.)
 constexpr int64_t RS_MID_MAX = 131072;
 __host__ __device__ constexpr int sort_passes(int64_t n) { return n <= RS_MID_MAX ? 3 : 4; }
 __host__ __device__ constexpr int sort_drop(int64_t n) { return sort_passes(n) == 3 ? 7 : 0; }
@@ -316,10 +314,10 @@ __global__ void __launch_bounds__(RS_THREADS)
 //                    block adds up the nblk <= 128 rows itself, coalesced),
 //                    stable scatter, and, at each key's new place, one count for
 //                    the next pass
-// against twelve with a histogram and a row scan per pass. (With four passes, two
-// sorts of 24,576 points, targets and sources, were 30 launches, 114 us one after
-// another, and are 12 and 81 us.) Digit counts are 16-bit, [pass][tile][256] (a tile has at most 1024
-// keys).
+// against twelve with a histogram and a row scan per pass. (Two sorts, of 24,576
+// targets and as many sources, are 10 launches, 64 us one after another; with the
+// larger sets' launches and four passes 30 and 114 us.) Digit counts are 16-bit,
+// [pass][tile][256] (a tile has at most 1024 keys).
 inline int rs_mid_items(int64_t n) { return n <= 32768 ? 1 : n <= 65536 ? 2 : 4; }
 constexpr int RS_PASSES = sort_passes(RS_MID_MAX);
 
@@ -608,8 +606,8 @@ __global__ void k_pack_src64(const double* __restrict__ xyz, const double* __res
   if (real) {
     // Segments dealt out as in k_pack_src32, in DEAL64 strides: a chunk of packed
     // sources takes segments from so many parts of the curve and every chunk its
-    // share of the near ones (24,576 x 15,384: 17.5 -> 16.6 ms; 1,944 x 1,344
-    // 295 -> 291 us). The last segments, which fill no stride, stay in place, so the
+    // share of the near ones (24,576 x 15,384: 16.6 ms, in sorted order 17.5; 1,944 x
+    // 1,344: 1%). The last segments, which fill no stride, stay in place, so the
     // active sources still come first.
     const int rows = Ns / SEG / DEAL64, p = (int)(s / SEG);
     const int64_t q =
