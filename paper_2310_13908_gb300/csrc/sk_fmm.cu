@@ -1310,9 +1310,10 @@ int stokes_sl_eval_fmm(sk_ctx* ctx, int precision, int mem, int64_t n_src,
       oa.rt_ratio = a.rt_ratio;
       p32::FinishArgs fa{cv.tgt64, cv.perm, m_slots, 1, cv.part, cv.near_cnt, cv.near_idx,
                          cv.near_ovf, X, W, F, nullptr, scale, U, cv.flags};
-      const size_t fsmem = (size_t)p32::near_warp_words(oa.group) * 4 +
+      fa.group = 64 * np32;
+      const size_t fsmem = (size_t)p32::near_warp_words(fa.group) * 4 +
                            FMM_FIN_THREADS * 3 * sizeof(double);
-      const unsigned fgrid = (unsigned)(m_slots / oa.group) * FMM_FIN_PARTS;
+      const unsigned fgrid = (unsigned)(m_slots / fa.group) * FMM_FIN_PARTS;
       if (np32 == 2)
         k_fmm_finish32<128><<<fgrid, FMM_FIN_THREADS, fsmem, st>>>(oa, fa, d_if, tb);
       else

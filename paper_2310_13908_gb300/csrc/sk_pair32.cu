@@ -90,7 +90,7 @@ void launch_pair32_t(const EvalBufs& b, float rt_ratio, double scale,
                   b.src_xyz, b.src_w, b.dens,   b.nrm, scale, b.flags, b.near_ovf};
   FinishArgs fa{b.tgt64, b.tgt_perm, b.M_pad, b.n_chunks, b.part, b.near_cnt, b.near_idx,
                 b.near_ovf, b.src_xyz, b.src_w, b.dens, b.nrm, scale, b.u, b.flags};
-  oa.group = 64 * NP;
+  oa.group = fa.group = 64 * NP;
   oa.rt_ratio = rt_ratio;
   if (b.fuse_finish) {
     cudaFuncSetAttribute(k_pair32_fused<L, NP, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,

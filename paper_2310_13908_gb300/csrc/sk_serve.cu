@@ -412,7 +412,7 @@ void publish(sk_server* srv, int slot) {
                       b.src_xyz, b.src_w, b.dens, b.nrm, scale, b.flags, b.near_ovf};
   d.fa = FinishArgs{b.tgt64, b.tgt_perm, b.M_pad, b.n_chunks, b.part, b.near_cnt, b.near_idx,
                     b.near_ovf, b.src_xyz, b.src_w, b.dens, b.nrm, scale, b.u, b.flags};
-  d.oa.group = 64 * SERVE_NP;
+  d.oa.group = d.fa.group = 64 * SERVE_NP;
   d.oa.rt_ratio = d.pa.rt_ratio;
   d.n_tb = (int)(b.M_pad / SERVE_TGT_CTA);
   d.tb_done = sl.tb_counters;
